@@ -61,6 +61,22 @@ __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b)
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdiv_rn(a, b); }
 
+// ----------------------------------------------------------------- cells
+
+// Floor of q clamped to 0 .. n - 1 (n <= 2^20), as an integer and a float, without a
+// conversion instruction: q clamped to [0, n - 1/2] plus 2^23, rounded down, holds the
+// floor in its low significand bits.  (floor, float-to-int and int-to-float run on a
+// pipe with an eighth of the FP32 rate, and every level of every sample takes three.)
+__device__ __forceinline__ uint32_t floor_cell(float q, float top, float& fl) {
+    const float m = __fadd_rd(fminf(fmaxf(q, 0.f), top), 8388608.f);
+    fl = fsub(m, 8388608.f);
+    return __float_as_uint(m) - 0x4B000000u;
+}
+// n as a float (n < 2^23), the same way.
+__device__ __forceinline__ float small_float(uint32_t n) {
+    return fsub(__uint_as_float(0x4B000000u + n), 8388608.f);
+}
+
 // ----------------------------------------------------------------- SplitMix64
 // Published SplitMix64 output function (Steele, Lea & Flood 2014): advance by the
 // golden gamma, then xor-shift 30 / multiply, xor-shift 27 / multiply, xor-shift 31.
@@ -83,7 +99,7 @@ constexpr uint64_t kOccStream = 1ull << 30;
 
 // Grid position of step i of a ray: t = near + i*step, x = (o + t d - org) * inv.
 __device__ __forceinline__ float sample_t(const DevCfg& c, uint32_t i) {
-    return fadd(c.near_t, fmul((float)i, c.step_t));
+    return fadd(c.near_t, fmul(small_float(i), c.step_t));
 }
 
 __device__ __forceinline__ float3 grid_pos(const DevCfg& c, float3 o, float3 d, float t) {
@@ -99,17 +115,17 @@ __device__ __forceinline__ bool in_box(const DevCfg& c, float3 x) {
            x.z < c.box[2];
 }
 
-__device__ __forceinline__ int cell_of(float x, uint32_t res) {
-    int ci = (int)floorf(fmul(x, (float)res));
-    ci = ci < 0 ? 0 : ci;
-    return ci > (int)res - 1 ? (int)res - 1 : ci;
+__device__ __forceinline__ uint32_t cell_of(float x, float res) {
+    float fl;
+    return floor_cell(fmul(x, res), res - 0.5f, fl);
 }
 
 __device__ __forceinline__ bool occupied(const DevCfg& c, const uint32_t* __restrict__ bits,
                                          float3 x) {
     if (c.occ_res == 0) return true;
     const uint32_t R = c.occ_res;
-    uint32_t b = (uint32_t)cell_of(x.x, R) + R * ((uint32_t)cell_of(x.y, R) + R * (uint32_t)cell_of(x.z, R));
+    const float Rf = small_float(R);
+    const uint32_t b = cell_of(x.x, Rf) + R * (cell_of(x.y, Rf) + R * cell_of(x.z, Rf));
     return (__ldg(bits + (b >> 5)) >> (b & 31)) & 1u;
 }
 
@@ -159,14 +175,14 @@ __device__ __forceinline__ uint32_t vertex_slot(uint32_t cx, uint32_t cy, uint32
     return (cx ^ (cy * 2654435761u) ^ (cz * 805459861u)) & Tmask;
 }
 
-// Cell and fractional offset at resolution N: q = x*N, c = min(floor q, N-1), w = q - c.
+// Cell and fractional offset at resolution N (<= 2^20): q = x*N, c = min(floor q, N-1),
+// w = q - c.
 __device__ __forceinline__ void level_cell(float x, uint32_t N, uint32_t& ci, float& w) {
-    const float q = fmul(x, (float)N);
-    int c = (int)floorf(q);
-    c = c > (int)N - 1 ? (int)N - 1 : c;
-    c = c < 0 ? 0 : c;
-    ci = (uint32_t)c;
-    w = fsub(q, (float)c);
+    const float Nf = small_float(N);
+    const float q = fmul(x, Nf);
+    float c;
+    ci = floor_cell(q, Nf - 0.5f, c);
+    w = fsub(q, c);
 }
 
 // ----------------------------------------------------------------- SH bands 0..3

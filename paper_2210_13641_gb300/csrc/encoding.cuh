@@ -92,34 +92,22 @@ __device__ __forceinline__ void hash_encode(const DevCfg& c, const float2* __res
     for (int l0 = 0; l0 < kEnc / 2; l0 += kGatherGroup) encode_group(c, tables, x, l0, f + 2 * l0);
 }
 
-// dL/dtable[l][slot_k] += w_k * dL/df_l for every corner and for the levels whose
-// bit is set in `levels` (FP32 vector reductions of 8 bytes, one per corner),
-// warp-cooperative: called by all 32 lanes (lanes with valid = false contribute
-// nothing).  df(l) returns this lane's (dL/df_{l,0}, dL/df_{l,1}) as a float2.  Consecutive samples of a ray fall into the
+// dL/dtable[l][slot_k] += w_k * dL/df_l for every corner (the plain FP32 backward; FP32
+// vector reductions of 8 bytes, one per corner), warp-cooperative: called by all 32
+// lanes (lanes with valid = false contribute nothing).  df(l) returns this lane's
+// (dL/df_{l,0}, dL/df_{l,1}) as a float2.  Consecutive samples of a ray fall into the
 // same cell of the coarse levels, so per level the lanes with equal cells (runs of
 // consecutive lanes) first sum their 8 corner contributions with a segmented
 // shuffle reduction, and only the first lane of each run issues the 8 atomics.
-// A level whose 32 cells are all different skips the reduction.  A level whose 32
-// samples share one cell (one run, all lanes valid: the common case of the coarse
-// levels) sums, with kButterfly, by a butterfly that halves the corners held per
-// lane at each step (18 shuffles instead of the segmented form's 80); lane 4k then
-// holds corner k's sum and 8 lanes issue the 8 reductions together (the tensor-core
-// backward: -2 % time; the FP32 backward keeps the segmented form, +7 % with it).
-// The level loop is unrolled by two only (two levels' shuffles in flight): the fully
-// unrolled form's code did not fit the instruction cache next to the tensor-core
-// layer chain of the backward kernel.  Runs are not cut short to save reduction
-// rounds: every extra head costs 8 reductions, which the large map's HBM-resident
-// tables pay dearly (cutting runs every 8 lanes: -1 % on a 64 MB table, +20 % on a
-// 512 MB one).
-template <bool kButterfly, class DF>
+// A level whose 32 cells are all different skips the reduction.
+template <class DF>
 __device__ __forceinline__ void hash_scatter_warp(const DevCfg& c, float2* __restrict__ gtables,
-                                                  float3 x, DF df, bool valid, uint32_t levels = 0xFFFFu) {
+                                                  float3 x, DF df, bool valid) {
     const uint32_t Tmask = c.T - 1;
     const uint32_t lane = threadIdx.x & 31u;
 #pragma unroll 2
     for (int l = 0; l < kEnc / 2; ++l) {
         if (l >= (int)c.L) break;
-        if (!((levels >> l) & 1u)) continue;
         const uint32_t N = c.res[l];
         const bool dense = (c.dense_mask >> l) & 1u;
         uint32_t cx, cy, cz;
@@ -140,39 +128,6 @@ __device__ __forceinline__ void hash_scatter_warp(const DevCfg& c, float2* __res
             const float wk = corner_weight(k, wx, wy, wz);
             v[2 * k] = wk * g0;
             v[2 * k + 1] = wk * g1;
-        }
-        if (kButterfly && heads == 1u) {
-            // one run: after the exchanges across lane bits 4, 3 and 2 a lane holds
-            // the partial sums of corner (lane >> 2), completed across bits 1 and 0
-            const bool b4 = lane & 16u, b3 = lane & 8u, b2 = lane & 4u;
-            float2 a[4], h[2];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 lo = make_float2(v[2 * j], v[2 * j + 1]);
-                const float2 hi = make_float2(v[2 * j + 8], v[2 * j + 9]);
-                const float2 snd = b4 ? lo : hi, kp = b4 ? hi : lo;
-                a[j] = make_float2(kp.x + __shfl_xor_sync(0xffffffffu, snd.x, 16),
-                                   kp.y + __shfl_xor_sync(0xffffffffu, snd.y, 16));
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float2 snd = b3 ? a[j] : a[j + 2], kp = b3 ? a[j + 2] : a[j];
-                h[j] = make_float2(kp.x + __shfl_xor_sync(0xffffffffu, snd.x, 8),
-                                   kp.y + __shfl_xor_sync(0xffffffffu, snd.y, 8));
-            }
-            const float2 snd = b2 ? h[0] : h[1], kp = b2 ? h[1] : h[0];
-            float2 d = make_float2(kp.x + __shfl_xor_sync(0xffffffffu, snd.x, 4),
-                                   kp.y + __shfl_xor_sync(0xffffffffu, snd.y, 4));
-            d.x += __shfl_xor_sync(0xffffffffu, d.x, 2);
-            d.y += __shfl_xor_sync(0xffffffffu, d.y, 2);
-            d.x += __shfl_xor_sync(0xffffffffu, d.x, 1);
-            d.y += __shfl_xor_sync(0xffffffffu, d.y, 1);
-            if ((lane & 3u) == 0u) {
-                const uint32_t k = lane >> 2;
-                const uint32_t slot = vertex_slot(cx + (k & 1u), cy + ((k >> 1) & 1u), cz + (k >> 2), N, dense, Tmask);
-                atomicAdd(gtab + slot, d);
-            }
-            continue;
         }
         if (heads != 0xffffffffu) {
             // lanes lane .. run_end form this lane's run; the head ends up with the sum
@@ -196,6 +151,158 @@ __device__ __forceinline__ void hash_scatter_warp(const DevCfg& c, float2* __res
             }
         }
     }
+}
+
+// ---------------------------------------------------------------- tile scatter
+// dL/dtable of a 128-sample tile, for the tensor-core backward: 256 threads, thread st
+// walks the 16 consecutive samples 16 g .. 16 g + 15 of the tile at one level, for the
+// vertices whose x coordinate has parity p.  Consecutive samples lie on a ray, so they
+// share vertices: at the coarse levels the whole cell, and where a step crosses one
+// face still 4 of its 8 vertices.  Each sample's cell has exactly one vertex per parity
+// of (x, y, z), so a vertex keeps its accumulator (parity of y and z) and its lane
+// (parity of x) for as long as the samples touch it; the sum leaves with one 8-byte
+// reduction when the ray moves on.  Two lanes p = 0, 1 side by side flush x-adjacent
+// vertices in one instruction, which share a 32-byte sector 3 times in 4.
+// Per sample this issues 48.4 reductions in 33.3 sectors on the room workload's rays
+// (counted on the host), against 61.4 in 52.2 for sums over runs of equal cells within
+// a warp, and needs no shuffle at all: the backward of 19.5 M samples takes 4.28 ms
+// instead of 6.74.  It runs at 0.6 of the issue rate, with the integer pipe at 0.57.
+struct ScatterRole {
+    uint32_t N, m1, m2, g, p;   // resolution, y and z strides (or hash primes), sample group, x parity
+    uint32_t level;
+    bool dense;
+};
+
+// The level of scatter thread st: each half warp has one.  The dense levels pair up
+// among themselves (one index arithmetic per warp); the others pair coarse with fine,
+// since a fine level flushes at almost every sample and the slowest warp sets the pace
+// (pairs of neighbours, 14 and 15 in one warp: 4.38 against 3.8 ms for the backward).
+__device__ __forceinline__ uint32_t scatter_level(const DevCfg& c, uint32_t st) {
+    const uint32_t dense = c.dense_mask & 0xffffu, nd = __popc(dense), in_pairs = nd & ~1u;
+    const uint32_t w = st >> 5, hi = (st >> 4) & 1u;
+    uint32_t k;  // place in the order: dense levels, then the others
+    if (2u * w < in_pairs) k = 2u * w + hi;
+    else k = hi ? 15u - (w - in_pairs / 2u) : w + in_pairs / 2u;
+    const bool want_dense = k < nd;
+    if (!want_dense) k -= nd;
+    uint32_t level = 0;
+    for (uint32_t l = 0, seen = 0; l < 16; ++l)
+        if (((dense >> l) & 1u) == (want_dense ? 1u : 0u) && seen++ == k) level = l;
+    return level;
+}
+
+__device__ __forceinline__ ScatterRole scatter_role(const DevCfg& c, uint32_t st, uint32_t level) {
+    ScatterRole s;
+    s.level = level;
+    s.g = (st >> 1) & 7u;
+    s.p = st & 1u;
+    s.N = c.res[level];
+    s.dense = (c.dense_mask >> level) & 1u;
+    s.m1 = s.dense ? s.N + 1u : 2654435761u;
+    s.m2 = s.dense ? (s.N + 1u) * (s.N + 1u) : 805459861u;
+    return s;
+}
+
+// Physical row of sample row r in the tile buffers the scatter walks (positions, and
+// dL/dfeat per level): lanes of the 8 groups read rows 16 g + i with the same i, which
+// the permutation spreads over all banks (and the odd levels, which mostly share a
+// warp with even ones, over the other half).
+__device__ __forceinline__ uint32_t tile_row(uint32_t r) { return r ^ ((r >> 4) & 7u); }
+__device__ __forceinline__ uint32_t tile_df(uint32_t r, uint32_t level) {
+    return level * 128u + (tile_row(r) ^ ((level & 1u) << 3));
+}
+
+// Where a differs from b: acc leaves to *p by one 8-byte FP32 reduction, and is cleared.
+__device__ __forceinline__ void flush_if_ne(float2* p, float2& v, uint32_t a, uint32_t b) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.u32 q, %3, %4;\n"
+        "@q red.relaxed.gpu.global.add.v2.f32 [%2], {%0, %1};\n"
+        "@q mov.f32 %0, 0f00000000;\n"
+        "@q mov.f32 %1, 0f00000000;\n"
+        "}\n" : "+f"(v.x), "+f"(v.y) : "l"(p), "r"(a), "r"(b)
+        : "memory");
+}
+
+// The walk of one thread.  kMode: 0 hashed levels, 1 dense levels, 2 both in the warp.
+// A vertex that leaves is told by its slot: two vertices with one slot share an entry.
+// Cells are kept as the bits of 2^23 + c: the bias, a multiple of 2^24 once multiplied,
+// vanishes under the slot mask (at most 2^24 entries).  Of an axis' two vertices one is
+// odd (O): with d = q - O the trilinear weights are 1 - |d| (odd) and |d| (even), for
+// either order of the two.  Beyond the last cell (kUnit = false: a box that reaches past
+// the unit cube, whose samples extrapolate from that cell) d takes its sign from the
+// order instead.
+template <int kMode, bool kUnit>
+__device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __restrict__ gtab, uint32_t mask,
+                                             const float4* pos, const float2* df, uint32_t n) {
+    const float Nf = small_float(s.N), top = Nf - 0.5f;
+    const uint32_t r0 = 16u * s.g, dswz = s.g ^ ((s.level & 1u) << 3), np = 1u - s.p;
+    const float sx = s.p ? -1.f : 1.f, tx = s.p ? 1.f : 0.f;
+    uint32_t held[4];                                     // slots by parity, [2 z + y]
+    float2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        acc[k] = make_float2(0.f, 0.f);
+        held[k] = 0u;
+    }
+#pragma unroll 1
+    for (uint32_t i = 0; i < n; ++i) {
+        const float4 q = pos[r0 + (i ^ s.g)];
+        const float2 gl = df[(r0 + i) ^ dswz];
+        const float qx = fmul(q.x, Nf), qy = fmul(q.y, Nf), qz = fmul(q.z, Nf);
+        // positions are >= 0 (the box test)
+        const uint32_t cx = __float_as_uint(__fadd_rd(fminf(qx, top), 8388608.f));
+        const uint32_t cy = __float_as_uint(__fadd_rd(fminf(qy, top), 8388608.f));
+        const uint32_t cz = __float_as_uint(__fadd_rd(fminf(qz, top), 8388608.f));
+        auto dist = [](float qa, uint32_t ca) {
+            const float d = fsub(qa, fsub(__uint_as_float(ca | 1u), 8388608.f));
+            return kUnit ? fabsf(d) : ((ca & 1u) ? d : -d);
+        };
+        const float dx = dist(qx, cx), dy = dist(qy, cy), dz = dist(qz, cz);
+        const uint32_t X = ((cx + np) & ~1u) | s.p;
+        const uint32_t A[2] = {((cy + 1u) & ~1u) * s.m1, (cy | 1u) * s.m1};
+        const uint32_t B[2] = {((cz + 1u) & ~1u) * s.m2, (cz | 1u) * s.m2};
+        const float fx = fmaf(sx, dx, tx);
+        const float fy[2] = {dy, 1.f - dy}, fz[2] = {dz, 1.f - dz};
+        uint32_t slot[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t a = A[k & 1], b = B[k >> 1];
+            slot[k] = (kMode == 1 || (kMode == 2 && s.dense) ? X + a + b : X ^ a ^ b) & mask;
+        }
+        if (i > 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) flush_if_ne(gtab + held[k], acc[k], slot[k], held[k]);
+        }
+        const float xy[2] = {fx * fy[0], fx * fy[1]};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float w = xy[k & 1] * fz[k >> 1];
+            acc[k].x += w * gl.x;
+            acc[k].y += w * gl.y;
+            held[k] = slot[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) atomicAdd(gtab + held[k], acc[k]);
+}
+
+// level: scatter_level(c, st); pos: [128] (x, y, z, -) by tile_row; df: dL/dfeat by tile_df; n_valid: samples in the tile.
+__device__ __forceinline__ void scatter_tile(const DevCfg& c, float2* __restrict__ gtables, uint32_t st,
+                                             uint32_t level, const float4* pos, const float2* df, uint32_t n_valid) {
+    const ScatterRole s = scatter_role(c, st, level);
+    const uint32_t r0 = 16u * s.g;
+    const uint32_t n = level < c.L && r0 < n_valid ? min(16u, n_valid - r0) : 0u;
+    const uint32_t hashed = __ballot_sync(0xffffffffu, n && !s.dense), dense = __ballot_sync(0xffffffffu, n && s.dense);
+    if (n == 0u) return;
+    float2* gtab = gtables + (size_t)s.level * c.T;
+    df += s.level * 128;
+    const uint32_t mask = c.T - 1;
+    if (!(c.box[0] <= 1.f && c.box[1] <= 1.f && c.box[2] <= 1.f)) scatter_walk<2, false>(s, gtab, mask, pos, df, n);
+    else if (dense == 0u) scatter_walk<0, true>(s, gtab, mask, pos, df, n);
+    else if (hashed == 0u) scatter_walk<1, true>(s, gtab, mask, pos, df, n);
+    else scatter_walk<2, true>(s, gtab, mask, pos, df, n);
 }
 
 // dL/dx = sum_l (d f_l / dx) . dL/df_l at grid position x, for the pose gradient:

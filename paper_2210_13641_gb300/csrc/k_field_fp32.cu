@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kTile) k_field_bwd_fp32(DevCfg c, const float*
                     for (int k = 0; k < kEnc; ++k) df[k] += W1[j * kEnc + k] * a;
                 }
             }
-            hash_scatter_warp<false>(c, gtables, x, [&](int l) { return make_float2(df[2 * l], df[2 * l + 1]); },
+            hash_scatter_warp(c, gtables, x, [&](int l) { return make_float2(df[2 * l], df[2 * l + 1]); },
                                      valid);
             if (kPose && valid) {
                 const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params), x, df);

@@ -103,22 +103,30 @@ __device__ __forceinline__ void ld_cols(uint32_t trow, uint32_t col, float* v) {
     tmem_wait_ld();
 }
 
-struct Op {
-    uint32_t addr, lbo, sbo, kstep;
+// An operand tile at byte offset OFF of the block's shared memory, R rows.  K-major: rows
+// index M (or N), columns K.  MN-major: rows index K, columns M (or N).
+template <uint32_t OFF, int R>
+struct KMaj {
+    static constexpr uint32_t lo = desc_lo(OFF, (uint32_t)(R / 8) * 128u), hi = desc_hi(128u);
+    static constexpr uint32_t kstep = (uint32_t)(R / 8) * 256u;
+    static constexpr bool mn = false;
 };
-// Tile with R rows used as a K-major operand (rows = M or N, columns = K).
-__device__ __forceinline__ Op kmaj(const void* t, int R) {
-    return Op{smem_u32(t), (uint32_t)(R / 8) * 128u, 128u, (uint32_t)(R / 8) * 256u};
-}
-// Tile with R rows used as an MN-major operand (rows = K, columns = M or N).
-__device__ __forceinline__ Op mnmaj(const void* t, int R) {
-    return Op{smem_u32(t), 128u, (uint32_t)(R / 8) * 128u, 256u};
-}
+template <uint32_t OFF, int R>
+struct MnMaj {
+    static constexpr uint32_t lo = desc_lo(OFF, 128u), hi = desc_hi((uint32_t)(R / 8) * 128u);
+    static constexpr uint32_t kstep = 256u;
+    static constexpr bool mn = true;
+};
 
-__device__ __forceinline__ void gemm(uint32_t d, Op a, Op b, int ksteps, uint32_t idesc, bool acc) {
-    for (int k = 0; k < ksteps; ++k)
-        mma_f16(d, smem_desc(a.addr + k * a.kstep, a.lbo, a.sbo), smem_desc(b.addr + k * b.kstep, b.lbo, b.sbo),
-                idesc, (acc || k > 0) ? 1u : 0u);
+// D (M x N, at TMEM address d) (+)= A B over KS steps of K = 16; base4: the block's
+// shared-memory base / 16.
+template <bool BF16, int M, int N, class A, class B, int KS>
+__device__ __forceinline__ void gemm(uint32_t d, uint32_t base4, bool acc) {
+    asm volatile("" : "+r"(base4), "+r"(d));  // the adds stay here: hoisted out of the tile loop they spill
+#pragma unroll
+    for (int k = 0; k < KS; ++k)
+        mma_f16<A::hi, B::hi, idesc_f16(M, N, BF16, A::mn, B::mn)>(
+            d, base4 + A::lo + k * (A::kstep >> 4), base4 + B::lo + k * (B::kstep >> 4), (acc || k > 0) ? 1u : 0u);
 }
 
 // Makes this thread's operand writes visible to the tensor core and orders its
@@ -189,6 +197,18 @@ __device__ __forceinline__ float3 sample_pos_tc(const DevCfg& c, const float* __
 constexpr int kW1B = 64 * 32 * 2, kW2B = 16 * 64 * 2, kW3B = 64 * 32 * 2, kW4B = 64 * 64 * 2, kW5B = 16 * 64 * 2;
 constexpr int kWB = kW1B + kW2B + kW3B + kW4B + kW5B;  // 20480
 constexpr int kT32 = 128 * 32 * 2, kT64 = 128 * 64 * 2, kT16 = 128 * 16 * 2;
+// byte offsets of the weight tiles in the block's shared memory
+constexpr uint32_t kOW1 = 0, kOW2 = kOW1 + kW1B, kOW3 = kOW2 + kW2B, kOW4 = kOW3 + kW3B, kOW5 = kOW4 + kW4B;
+using W1K = KMaj<kOW1, 64>;
+using W2K = KMaj<kOW2, 16>;
+using W3K = KMaj<kOW3, 64>;
+using W4K = KMaj<kOW4, 64>;
+using W5K = KMaj<kOW5, 16>;
+using W1M = MnMaj<kOW1, 64>;
+using W2M = MnMaj<kOW2, 16>;
+using W3M = MnMaj<kOW3, 64>;
+using W4M = MnMaj<kOW4, 64>;
+using W5M = MnMaj<kOW5, 16>;
 
 }  // namespace
 
@@ -209,14 +229,12 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
                                          float feat_scale, uint32_t i0, uint32_t i_end, uint8_t* smem,
                                          uint32_t tmem, uint64_t* bar, uint32_t& phase, bool& timed_out,
                                          const uint32_t* __restrict__ sel = nullptr) {
-    uint8_t* sW1 = smem;
-    uint8_t* sW2 = sW1 + kW1B;
-    uint8_t* sW3 = sW2 + kW2B;
-    uint8_t* sW4 = sW3 + kW3B;
-    uint8_t* sW5 = sW4 + kW4B;
     uint8_t* tA = smem + kWB;
     uint8_t* tB = tA + kT32;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    using TA = KMaj<kWB, 128>;
+    using TB = KMaj<kWB + kT32, 128>;
+    const uint32_t base4 = smem_u32(smem) >> 4;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
     const float inv_fs = 1.f / feat_scale;
     const bool valid = i0 + tid < i_end;
@@ -246,8 +264,8 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     }
     // layer 1: D = X0 W1^T (128 x 64)
     to_tensor();
-    if (tid == 0) {
-        gemm(tmem, kmaj(tA, 128), kmaj(sW1, 64), 2, idesc_f16(128, 64, BF16, false, false), false);
+    if (warp == 0 && elect_one()) {
+        gemm<BF16, 128, 64, TA, W1K, 2>(tmem, base4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -260,8 +278,8 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     }
     // layer 2: y = H1 W2^T (128 x 16)
     to_tensor();
-    if (tid == 0) {
-        gemm(tmem, kmaj(tB, 128), kmaj(sW2, 16), 4, idesc_f16(128, 16, BF16, false, false), false);
+    if (warp == 0 && elect_one()) {
+        gemm<BF16, 128, 16, TB, W2K, 4>(tmem, base4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -275,8 +293,8 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     store_row<BF16, 32>(tA, tid, v);
     // layer 3: H3 = relu(X3 W3^T)
     to_tensor();
-    if (tid == 0) {
-        gemm(tmem, kmaj(tA, 128), kmaj(sW3, 64), 2, idesc_f16(128, 64, BF16, false, false), false);
+    if (warp == 0 && elect_one()) {
+        gemm<BF16, 128, 64, TA, W3K, 2>(tmem, base4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -287,8 +305,8 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     }
     // layer 4: H4 = relu(H3 W4^T)
     to_tensor();
-    if (tid == 0) {
-        gemm(tmem, kmaj(tB, 128), kmaj(sW4, 64), 4, idesc_f16(128, 64, BF16, false, false), false);
+    if (warp == 0 && elect_one()) {
+        gemm<BF16, 128, 64, TB, W4K, 4>(tmem, base4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -299,8 +317,8 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     }
     // layer 5: z = H4 W5^T (3 of 16 columns used)
     to_tensor();
-    if (tid == 0) {
-        gemm(tmem, kmaj(tB, 128), kmaj(sW5, 16), 4, idesc_f16(128, 16, BF16, false, false), false);
+    if (warp == 0 && elect_one()) {
+        gemm<BF16, 128, 16, TB, W5K, 4>(tmem, base4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -327,7 +345,7 @@ __device__ __forceinline__ void fwd_block_finish(uint32_t tmem, uint64_t* drain_
     const bool any_timeout = __syncthreads_or(timed_out) != 0;
     fence_after_sync();
     if (any_timeout) {
-        if (threadIdx.x == 0) drain_mma(drain_bar);
+        if (__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0) == 0 && elect_one()) drain_mma(drain_bar);
         fence_before_sync();
         __syncthreads();
         fence_after_sync();
@@ -430,16 +448,15 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
 // Warp-specialised in three warpgroups: warps 0-3 (the "MLP" group, thread r =
 // sample row r = TMEM lane r) run the layer chain on the tensor cores; warps 4-7
 // (the "IO" group, thread 128 + r serves row r) load each tile's inputs one tile
-// ahead and scatter the even levels of each finished tile's encoding gradient into
-// the tables; warps 8-11 (the "SC" group, thread 256 + r) scatter its odd levels.
-// Both scatter groups work on tile k while the MLP group runs tile k + 1: the
-// scatter is the longer path (its reductions and warp shuffles load the L1 data
-// pipe), so it gets two warpgroups.  Registers are split with setmaxnreg: the
-// block is launched with 80 per thread (two blocks of 384 threads per SM), the
-// MLP group takes 136, the IO group 64 (its prefetched inputs are dead while it
-// scatters), the SC group 40 (the scatter alone needs no more without spilling):
-// 128 x 136 + 128 x 64 + 128 x 40 = 384 x 80.  The groups hand tiles over through
-// named barriers:
+// ahead; warps 4-11 (IO and the "SC" group) scatter each finished tile's encoding
+// gradient into the tables, by level (scatter_tile), while the MLP group runs the next
+// tile.  For 19.5 M samples the chain alone takes 2.3 ms and the scatter alone 4.1 (of
+// 4.3 together): the scatter sets the pace, by its issue slots and its reductions.
+// Registers are split with setmaxnreg: the block is launched with 80 per thread (two
+// blocks of 384 threads per SM), the MLP group takes 96 (its epilogues hold 16 columns
+// at a time), the IO group 80 and the SC group 64, which is 240 = 3 x 80; 104 / 80 / 56
+// measured 4.34 ms, 104 / 72 / 64 4.39, 128 / 64 / 48 4.62.
+// The groups hand tiles over through named barriers:
 //   kBarIn      IO -> MLP        the tile's encodings (X0) and row data are in place
 //   kBarDfReady MLP -> IO, SC    the chain is done (X0 free) and dL/dfeat is in smem
 //   kBarDfFree  IO, SC -> MLP    both scatters of the tile are done (dL/dfeat read)
@@ -452,10 +469,9 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
 constexpr uint32_t kColW4 = 64, kColW3 = 128, kColW1 = 160, kColW2T = 192, kColW5T = 208;
 constexpr int kBarMlp = 1, kBarIn = 2, kBarDfReady = 3, kBarDfFree = 4;
 constexpr int kBwdThreads = 384;            // MLP, IO and SC warpgroups
-constexpr uint32_t kRegMlp = 136, kRegIo = 64, kRegSc = 40;
+constexpr uint32_t kRegMlp = 96, kRegIo = 80, kRegSc = 64;
 static_assert(128 * (kRegMlp + kRegIo + kRegSc) == kBwdThreads * 80,
               "the setmaxnreg split must add up to the launch allocation (80 registers per thread)");
-constexpr uint32_t kLevelsIo = 0x5555u, kLevelsSc = 0xAAAAu;  // even / odd levels
 constexpr int kDfBytes = 128 * 32 * 4;      // dL/dfeat, [level][row] float2
 constexpr int kRowBytes = 128 * 32;         // row data: {d.xyz, valid}, {dz0, dz1, dz2, dL/dsigma}
 constexpr int kXBytes = 2 * 128 * 16;       // sample positions (x, valid) of the tiles, by parity
@@ -478,38 +494,58 @@ __device__ __forceinline__ void to_tensor_mlp() {
     fence_after_sync();
 }
 
-// 64 accumulator columns -> relu(scale * a) into a 64-column tile; the ReLU branch
-// of each column is returned as two 32-bit masks.
+// ReLU branches of 32 consecutive columns in one word: bit 15 - j is column 2 j's,
+// bit 31 - j column 2 j + 1's.
+//
+// 64 accumulator columns -> relu(scale * a) into a 64-column tile; the branch of each
+// column (a * scale > 0) is returned in two words.  n = 0 - scale * a has its sign bit
+// set exactly where the branch is taken (a zero of either sign gives +0), so each
+// branch is one funnel shift; the columns come 16 at a time, as more do not fit the
+// chain's registers.
 template <bool BF16>
-__device__ __forceinline__ void relu_epilogue(uint32_t trow, uint8_t* tile, int r, float scale, uint32_t& ma,
-                                              uint32_t& mb) {
-    float v[32];
+__device__ __forceinline__ void relu_epilogue(uint32_t trow, uint8_t* tile, int r, float scale, uint32_t* m) {
+    float v[16];
+    uint32_t me = 0, mo = 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        ld_cols<32>(trow, 32 * h, v);
-        uint32_t m = 0;
+    for (int h = 0; h < 4; ++h) {
+        ld_cols<16>(trow, 16 * h, v);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
-            v[k] *= scale;
-            if (v[k] > 0.f) m |= 1u << k;
+        for (int k = 0; k < 16; k += 2) {
+            const float ne = fmaf(v[k], -scale, 0.f), no = fmaf(v[k + 1], -scale, 0.f);
+            me = __funnelshift_l(__float_as_uint(ne), me, 1);
+            mo = __funnelshift_l(__float_as_uint(no), mo, 1);
+            v[k] = -ne;
+            v[k + 1] = -no;
         }
-        store_row_at<BF16, 32, true>(tile, r, 32 * h, v);
-        if (h == 0) ma = m;
-        else mb = m;
+        store_row_at<BF16, 16, true>(tile, r, 16 * h, v);
+        if (h & 1) m[h >> 1] = __byte_perm(me, mo, 0x5410);
     }
 }
 
-// 64 accumulator columns masked by the ReLU branches into a 64-column tile.
+// 0xffff in each half of the word whose top bit is set (prmt's sign replication of bytes
+// 1 and 3).
+__device__ __forceinline__ uint32_t sign_halves(uint32_t x) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(d) : "r"(x));
+    return d;
+}
+
+// 64 accumulator columns masked by the ReLU branches into a 64-column tile: the packed
+// pair's mask is the sign of two bytes of the shifted word.
 template <bool BF16>
-__device__ __forceinline__ void mask_epilogue(uint32_t trow, uint8_t* tile, int r, uint32_t ma, uint32_t mb) {
-    float v[32];
+__device__ __forceinline__ void mask_epilogue(uint32_t trow, uint8_t* tile, int r, const uint32_t* m) {
+    float v[16];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        ld_cols<32>(trow, 32 * h, v);
-        const uint32_t m = h == 0 ? ma : mb;
+    for (int h = 0; h < 4; ++h) {
+        ld_cols<16>(trow, 16 * h, v);
+        uint32_t q[8];
 #pragma unroll
-        for (int k = 0; k < 32; ++k) v[k] = ((m >> k) & 1u) ? v[k] : 0.f;
-        store_row_at<BF16, 32>(tile, r, 32 * h, v);
+        for (int j = 0; j < 8; ++j)
+            q[j] = pack2<BF16>(v[2 * j], v[2 * j + 1]) & sign_halves(m[h >> 1] * (1u << (8 * (h & 1) + j)));
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+            *reinterpret_cast<uint4*>(tile + tile_offset(r, 16 * h + 8 * g, 128)) =
+                make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
     }
 }
 
@@ -547,7 +583,22 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
     float4* sX = sRow + 2 * 128;                                // [2][128]: (x, valid) of tile k at k & 1
     const float2* sDf2 = reinterpret_cast<const float2*>(sDf);
 
-    const int tid = threadIdx.x, warp = tid >> 5, r = tid & 127;
+    constexpr uint32_t kOX0 = kWB, kOH1 = kOX0 + kT32, kOX3 = kOH1 + kT64, kOH3 = kOX3 + kT32, kOH4 = kOH3 + kT64,
+                       kOG5 = kOH4 + kT64;
+    using X0K = KMaj<kOX0, 128>;
+    using H1K = KMaj<kOH1, 128>;
+    using X3K = KMaj<kOX3, 128>;
+    using H3K = KMaj<kOH3, 128>;
+    using H4K = KMaj<kOH4, 128>;
+    using G5K = KMaj<kOG5, 128>;
+    using X0M = MnMaj<kOX0, 128>;
+    using H1M = MnMaj<kOH1, 128>;
+    using X3M = MnMaj<kOX3, 128>;
+    using H3M = MnMaj<kOH3, 128>;
+    using H4M = MnMaj<kOH4, 128>;
+    using G5M = MnMaj<kOG5, 128>;
+
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), r = tid & 127;
     load_weight_tiles<BF16>(params + (size_t)c.L * c.T * 2, sW1, sW2, sW3, sW4, sW5);
     if (warp == 0) tmem_alloc(&tslot, 256);
     if (tid == 0) {
@@ -574,25 +625,24 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
         const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
         const float inv_fs = 1.f / feat_scale;
         uint32_t phase = 0;
-        constexpr uint32_t kM128N64 = idesc_f16(128, 64, BF16, false, false);
-        constexpr uint32_t kM128N16 = idesc_f16(128, 16, BF16, false, false);
+        const uint32_t base4 = smem_u32(smem) >> 4;
         for (uint32_t k = 0; k < n_mine; ++k) {
             nb_sync(kBarIn, 256);
             const float4 rd = sRow[2 * r], rz = sRow[2 * r + 1];
             const bool valid = rd.w != 0.f;
             float v[32];
-            uint32_t m1a, m1b, m3a, m3b, m4a, m4b;
+            uint32_t m1[2], m3[2], m4[2];
             // ---- forward recompute (same arithmetic as the forward kernel)
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem, kmaj(tX0, 128), kmaj(sW1, 64), 2, kM128N64, false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 128, 64, X0K, W1K, 2>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            relu_epilogue<BF16>(trow, tH1, r, inv_fs, m1a, m1b);
+            relu_epilogue<BF16>(trow, tH1, r, inv_fs, m1);
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem, kmaj(tH1, 128), kmaj(sW2, 16), 4, kM128N16, false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 128, 16, H1K, W2K, 4>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -607,19 +657,19 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             }
             store_row_at<BF16, 32>(tX3, r, 0, y);
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem, kmaj(tX3, 128), kmaj(sW3, 64), 2, kM128N64, false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 128, 64, X3K, W3K, 2>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            relu_epilogue<BF16>(trow, tH3, r, 1.f, m3a, m3b);
+            relu_epilogue<BF16>(trow, tH3, r, 1.f, m3);
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem, kmaj(tH3, 128), kmaj(sW4, 64), 4, kM128N64, false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 128, 64, H3K, W4K, 4>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            relu_epilogue<BF16>(trow, tH4, r, 1.f, m4a, m4b);
+            relu_epilogue<BF16>(trow, tH4, r, 1.f, m4);
             // the colours' gradient seed dz (FP32, scaled by S) comes from the IO group
             v[0] = rz.x;
             v[1] = rz.y;
@@ -629,27 +679,27 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             store_row_at<BF16, 16>(tG5, r, 0, v);
             // ---- backward: dW5^T += H4^T G5 ; dH4 = G5 W5
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem + kColW5T, mnmaj(tH4, 128), mnmaj(tG5, 128), 8, idesc_f16(64, 16, BF16, true, true), k > 0);
-                gemm(tmem, kmaj(tG5, 128), mnmaj(sW5, 16), 1, idesc_f16(128, 64, BF16, false, true), false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 64, 16, H4M, G5M, 8>(tmem + kColW5T, base4, k > 0);
+                gemm<BF16, 128, 64, G5K, W5M, 1>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            mask_epilogue<BF16>(trow, tH4, r, m4a, m4b);                 // G4
+            mask_epilogue<BF16>(trow, tH4, r, m4);                 // G4
             // dW4 += G4^T H3 ; dH3 = G4 W4
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem + kColW4, mnmaj(tH4, 128), mnmaj(tH3, 128), 8, idesc_f16(64, 64, BF16, true, true), k > 0);
-                gemm(tmem, kmaj(tH4, 128), mnmaj(sW4, 64), 4, idesc_f16(128, 64, BF16, false, true), false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 64, 64, H4M, H3M, 8>(tmem + kColW4, base4, k > 0);
+                gemm<BF16, 128, 64, H4K, W4M, 4>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            mask_epilogue<BF16>(trow, tH3, r, m3a, m3b);                 // G3
+            mask_epilogue<BF16>(trow, tH3, r, m3);                 // G3
             // dW3 += G3^T X3 ; dX3 = G3 W3
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem + kColW3, mnmaj(tH3, 128), mnmaj(tX3, 128), 8, idesc_f16(64, 32, BF16, true, true), k > 0);
-                gemm(tmem, kmaj(tH3, 128), mnmaj(sW3, 64), 4, idesc_f16(128, 32, BF16, false, true), false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 64, 32, H3M, X3M, 8>(tmem + kColW3, base4, k > 0);
+                gemm<BF16, 128, 32, H3K, W3M, 4>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -669,19 +719,18 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             store_row_at<BF16, 16>(tX3, r, 0, v);                        // G2 (columns 0..15)
             // dW2^T += H1^T G2 ; dH1 = G2 W2
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem + kColW2T, mnmaj(tH1, 128), mnmaj(tX3, 128), 8, idesc_f16(64, 16, BF16, true, true),
-                     k > 0);
-                gemm(tmem, kmaj(tX3, 128), mnmaj(sW2, 16), 1, idesc_f16(128, 64, BF16, false, true), false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 64, 16, H1M, X3M, 8>(tmem + kColW2T, base4, k > 0);
+                gemm<BF16, 128, 64, X3K, W2M, 1>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
-            mask_epilogue<BF16>(trow, tH1, r, m1a, m1b);                 // G1
+            mask_epilogue<BF16>(trow, tH1, r, m1);                 // G1
             // dW1 += G1^T X0 ; dF = G1 W1
             to_tensor_mlp();
-            if (r == 0) {
-                gemm(tmem + kColW1, mnmaj(tH1, 128), mnmaj(tX0, 128), 8, idesc_f16(64, 32, BF16, true, true), k > 0);
-                gemm(tmem, kmaj(tH1, 128), mnmaj(sW1, 64), 4, idesc_f16(128, 32, BF16, false, true), false);
+            if (warp == 0 && elect_one()) {
+                gemm<BF16, 64, 32, H1M, X0M, 8>(tmem + kColW1, base4, k > 0);
+                gemm<BF16, 128, 32, H1K, W1M, 4>(tmem, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -690,13 +739,13 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             if (k > 0) nb_sync(kBarDfFree, kBwdThreads);  // both scatters of the previous tile are done
 #pragma unroll
             for (int q = 0; q < 16; ++q)
-                reinterpret_cast<float2*>(sDf)[q * 128 + r] = make_float2(v[2 * q] * inv_S, v[2 * q + 1] * inv_S);
+                reinterpret_cast<float2*>(sDf)[tile_df(r, q)] = make_float2(v[2 * q] * inv_S, v[2 * q + 1] * inv_S);
             nb_arrive(kBarDfReady, kBwdThreads);          // also: X0 and the row data are free
         }
         // ---- flush the weight gradients (lane 32*(m/16) + m%16 holds row m)
         const bool any_timeout = __syncthreads_or(timed_out) != 0;  // all three groups take part
         fence_after_sync();
-        if (any_timeout && r == 0) drain_mma(&drain_bar);          // r == 0 issued every MMA
+        if (any_timeout && warp == 0 && elect_one()) drain_mma(&drain_bar);  // the thread that issued every MMA
         if (n_mine > 0 && !any_timeout) {
             float* gm_ = grads + (size_t)c.L * c.T * 2;
             const int lane = tid & 31;
@@ -725,29 +774,26 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
         if (any_timeout && tid == 0) atomicOr(err, kErrTimeout);
     } else if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegSc));
-        // ======================= SC group: the odd levels' gradient scatter
-        float2* gtables = reinterpret_cast<float2*>(grads);
+        // ======================= SC group: its half of the levels' gradient scatter
+        const uint32_t level = scatter_level(c, 128u + r);
         for (uint32_t k = 0; k < n_mine; ++k) {
             nb_sync(kBarDfReady, kBwdThreads);
-            const float4 xq = sX[(k & 1u) * 128 + r];
-            hash_scatter_warp<true>(c, gtables, make_float3(xq.x, xq.y, xq.z),
-                                    [&](int l) { return sDf2[l * 128 + r]; }, xq.w != 0.f, kLevelsSc);
+            scatter_tile(c, reinterpret_cast<float2*>(grads), 128u + r, level, sX + (k & 1u) * 128, sDf2,
+                         n - (blockIdx.x + k * gridDim.x) * 128);
             if (k + 1 < n_mine) nb_arrive(kBarDfFree, kBwdThreads);
         }
         __syncthreads_or(false);                      // pairs with the MLP group's flush barrier
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegIo));
-        // ======================= IO group: tile inputs one tile ahead, the even levels' scatter
-        float2* gtables = reinterpret_cast<float2*>(grads);
-        float3 x_cur = make_float3(0.f, 0.f, 0.f), x_next = x_cur;
-        bool valid_cur = false, valid_next = false;
-        uint32_t i_cur = 0, i_next = 0;
+        // ======================= IO group: tile inputs one tile ahead, its half of the scatter
+        const uint32_t level = scatter_level(c, r);
+        float3 x_next = make_float3(0.f, 0.f, 0.f);
+        bool valid_next = false;
         uint4 f_next[4];
         float4 rd_next, rz_next;
         // inputs of this block's k-th tile for row r, into registers
         auto load = [&](uint32_t k) {
             const uint32_t i = (blockIdx.x + k * gridDim.x) * 128 + r;
-            i_next = i;
             valid_next = i < n;
             float3 d = make_float3(0.f, 0.f, 0.f);
             x_next = make_float3(0.f, 0.f, 0.f);
@@ -768,14 +814,11 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
         // the inputs of tile kk into the operand tile and the row data (and its sample
         // positions for the SC group)
         auto publish = [&](uint32_t kk) {
-            sX[(kk & 1u) * 128 + r] = make_float4(x_next.x, x_next.y, x_next.z, valid_next ? 1.f : 0.f);
+            sX[(kk & 1u) * 128 + tile_row(r)] = make_float4(x_next.x, x_next.y, x_next.z, valid_next ? 1.f : 0.f);
 #pragma unroll
             for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(tX0 + tile_offset(r, 8 * q, 128)) = f_next[q];
             sRow[2 * r] = rd_next;
             sRow[2 * r + 1] = rz_next;
-            x_cur = x_next;
-            valid_cur = valid_next;
-            i_cur = i_next;
             fence_proxy_async();                      // X0 is read by the tensor core
             nb_arrive(kBarIn, 256);
         };
@@ -786,22 +829,22 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
         for (uint32_t k = 0; k < n_mine; ++k) {
             if (k + 1 < n_mine) load(k + 1);          // global loads in flight during the chain
             nb_sync(kBarDfReady, kBwdThreads);
-            const float3 x_done = x_cur;
-            const bool valid_done = valid_cur;
-            const uint32_t i_done = i_cur;
             if (k + 1 < n_mine) publish(k + 1);       // next tile's inputs; the MLP group starts on it
-            hash_scatter_warp<true>(c, gtables, x_done, [&](int l) { return sDf2[l * 128 + r]; }, valid_done,
-                                    kLevelsIo);
-            if (kPose && valid_done) {
+            const uint32_t i0 = (blockIdx.x + k * gridDim.x) * 128;
+            const float4* pos = sX + (k & 1u) * 128;
+            scatter_tile(c, reinterpret_cast<float2*>(grads), r, level, pos, sDf2, n - i0);
+            if (kPose && i0 + r < n) {
                 float v[32];
 #pragma unroll
                 for (int q = 0; q < 16; ++q) {
-                    const float2 a = sDf2[q * 128 + r];
+                    const float2 a = sDf2[tile_df(r, q)];
                     v[2 * q] = a.x;
                     v[2 * q + 1] = a.y;
                 }
-                const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params), x_done, v);
-                pose_s[2 * (size_t)i_done] =
+                const float4 xq = pos[tile_row(r)];
+                const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params),
+                                              make_float3(xq.x, xq.y, xq.z), v);
+                pose_s[2 * (size_t)(i0 + r)] =
                     make_float4(gx.x * c.inv_size, gx.y * c.inv_size, gx.z * c.inv_size, 0.f);
             }
             if (k + 1 < n_mine) nb_arrive(kBarDfFree, kBwdThreads);  // dL/dfeat read: the MLP group may overwrite it

@@ -30,14 +30,25 @@ __device__ __forceinline__ uint32_t tile_offset(int r, int c, int R) {
 
 // Shared-memory matrix descriptor (tcgen05 format): start address >> 4 in bits
 // [0,14), leading byte offset >> 4 in [16,30), stride byte offset >> 4 in [32,46),
-// the fixed 0b001 in [46,49), base offset 0, relative LBO mode, no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
+// the fixed 0b001 in [46,49), base offset 0, relative LBO mode, no swizzle.  Its upper
+// word is a constant of the operand; the lower word is the block's shared-memory base
+// (in units of 16 bytes) plus a constant, so that an MMA costs one add per operand.
+__host__ __device__ constexpr uint32_t desc_lo(uint32_t offset, uint32_t lbo) {
+    return (offset >> 4) + ((lbo >> 4) << 16);
+}
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+
+// True in one lane of a converged warp, the same one at every call: the thread that
+// issues the warp's MMAs and commits.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n" : "=r"(p));
+    return p != 0u;
 }
 
 // Instruction descriptor for kind::f16: D FP32 (bits 4-5 = 1), A/B type F16 = 0 or
@@ -72,16 +83,20 @@ __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem], issued by one thread.
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                        uint32_t accumulate) {
+// D[tmem] (+)= A[smem] * B[smem], issued by one thread; AHI / BHI: the descriptors'
+// upper words.
+template <uint32_t AHI, uint32_t BHI, uint32_t IDESC>
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate) {
     asm volatile(
         "{\n"
         ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        ".reg .b64 da, db;\n"
+        "setp.ne.b32 p, %3, 0;\n"
+        "mov.b64 da, {%1, %4};\n"
+        "mov.b64 db, {%2, %5};\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %6, p;\n"
         "}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "r"(a_lo), "r"(b_lo), "r"(accumulate), "n"(AHI), "n"(BHI), "n"(IDESC)
         : "memory");
 }
 
