@@ -17,8 +17,7 @@ __device__ __forceinline__ float corner_weight(int k, float wx, float wy, float 
 // aligned 16-byte chunk (two float2 entries) exactly when s' = s ^ 1: in a hashed
 // level that holds whenever cx is even (the x coordinate enters the hash by xor with
 // prime 1), in a dense level whenever s is even.  The encoding reads such a pair
-// with one 16-byte load.  (The gradient scatter keeps one 8-byte reduction per
-// corner: 16-byte reductions of the shared pairs made the backward slower.)
+// with one 16-byte load.
 __device__ __forceinline__ bool x_pair_shared(uint32_t s0, uint32_t s1) { return (s0 ^ s1) == 1u; }
 
 // Features of levels l0 .. l0 + kGatherGroup - 1 of grid position x into
@@ -92,69 +91,8 @@ __device__ __forceinline__ void hash_encode(const DevCfg& c, const float2* __res
     for (int l0 = 0; l0 < kEnc / 2; l0 += kGatherGroup) encode_group(c, tables, x, l0, f + 2 * l0);
 }
 
-// dL/dtable[l][slot_k] += w_k * dL/df_l for every corner (the plain FP32 backward; FP32
-// vector reductions of 8 bytes, one per corner), warp-cooperative: called by all 32
-// lanes (lanes with valid = false contribute nothing).  df(l) returns this lane's
-// (dL/df_{l,0}, dL/df_{l,1}) as a float2.  Consecutive samples of a ray fall into the
-// same cell of the coarse levels, so per level the lanes with equal cells (runs of
-// consecutive lanes) first sum their 8 corner contributions with a segmented
-// shuffle reduction, and only the first lane of each run issues the 8 atomics.
-// A level whose 32 cells are all different skips the reduction.
-template <class DF>
-__device__ __forceinline__ void hash_scatter_warp(const DevCfg& c, float2* __restrict__ gtables,
-                                                  float3 x, DF df, bool valid) {
-    const uint32_t Tmask = c.T - 1;
-    const uint32_t lane = threadIdx.x & 31u;
-#pragma unroll 2
-    for (int l = 0; l < kEnc / 2; ++l) {
-        if (l >= (int)c.L) break;
-        const uint32_t N = c.res[l];
-        const bool dense = (c.dense_mask >> l) & 1u;
-        uint32_t cx, cy, cz;
-        float wx, wy, wz;
-        level_cell(x.x, N, cx, wx);
-        level_cell(x.y, N, cy, wy);
-        level_cell(x.z, N, cz, wz);
-        float2* gtab = gtables + (size_t)l * c.T;
-        const float2 gl = df(l);
-        const float g0 = valid ? gl.x : 0.f, g1 = valid ? gl.y : 0.f;
-        const uint64_t key = valid ? (((uint64_t)cz << 42) | ((uint64_t)cy << 21) | cx) : ~(uint64_t)lane;
-        const uint64_t prev = __shfl_up_sync(0xffffffffu, key, 1);
-        const bool head = lane == 0 || prev != key;
-        const uint32_t heads = __ballot_sync(0xffffffffu, head);
-        float v[16];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float wk = corner_weight(k, wx, wy, wz);
-            v[2 * k] = wk * g0;
-            v[2 * k + 1] = wk * g1;
-        }
-        if (heads != 0xffffffffu) {
-            // lanes lane .. run_end form this lane's run; the head ends up with the sum
-            const uint32_t above = (lane == 31u) ? 0u : (heads & ~((2u << lane) - 1u));
-            const uint32_t run_end = above ? (uint32_t)(__ffs(above) - 2) : 31u;
-            const uint32_t max_len = __reduce_max_sync(0xffffffffu, head ? run_end - lane + 1u : 1u);
-            for (uint32_t off = 1; off < max_len; off <<= 1) {
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const float o = __shfl_down_sync(0xffffffffu, v[q], off);
-                    if (lane + off <= run_end) v[q] += o;
-                }
-            }
-        }
-        if (head && valid) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t slot = vertex_slot(cx + (k & 1), cy + ((k >> 1) & 1), cz + ((k >> 2) & 1), N,
-                                                  dense, Tmask);
-                atomicAdd(gtab + slot, make_float2(v[2 * k], v[2 * k + 1]));
-            }
-        }
-    }
-}
-
 // ---------------------------------------------------------------- tile scatter
-// dL/dtable of a 128-sample tile, for the tensor-core backward: 256 threads, thread st
+// dL/dtable of a 128-sample tile (both backward kernels): 256 threads, thread st
 // walks the 16 consecutive samples 16 g .. 16 g + 15 of the tile at one level, for the
 // vertices whose x coordinate has parity p.  Consecutive samples lie on a ray, so they
 // share vertices: at the coarse levels the whole cell, and where a step crosses one

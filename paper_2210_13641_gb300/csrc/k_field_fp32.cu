@@ -2,12 +2,8 @@
 // density MLP (sigma = exp(h_0)), SH view encoding and colour MLP (sigmoid) forward
 // (steps a3-a6), and the recomputing backward pass (steps a10-a11).
 //
-// Forward: one thread per sample, weights in shared memory.  Backward: tiles of
-// 128 samples per 128-thread block; each thread recomputes its sample's activations
-// into a shared-memory row, the block then forms the weight-gradient tile products
-// (sum over the tile's samples), and every thread scatters its encoding gradient into
-// the tables with FP32 atomics.  Weight gradients stay in shared memory across the
-// tiles a persistent block visits and are flushed with one atomic per weight.
+// Forward: one thread per sample, weights in shared memory.  Backward: tiles of 128
+// samples whose activations are recomputed into shared memory (see there).
 #include "encoding.cuh"
 #include "internal.h"
 
@@ -142,50 +138,165 @@ void launch_field_fwd_fp32_sel(const DevCfg& c, const float* params, const uint3
 }
 
 // ------------------------------------------------------------------ backward
+// A 256-thread block per SM walks tiles of 128 samples.  A tile's activations sit in
+// shared memory, one row of 260 floats per sample, and every layer is a phase between
+// block barriers:
+//  - layer products (forward recompute and data gradients): a thread takes 4 samples and
+//    an eighth of the outputs (4 x 8 sums in registers), 4 inputs at a time: 4 16-byte
+//    loads of activations and 8 of weights, which all lanes share, for 128 multiply-adds.
+//    The recompute sums in the forward kernel's order, so its ReLU branches are the
+//    forward's, bit for bit;
+//  - weight gradients: a thread owns 8 rows and 4 columns of each weight matrix for a part
+//    of the samples (3 16-byte loads for 32 multiply-adds); its sums stay in registers over
+//    all tiles of the block and meet in shared memory at its end;
+//  - the encoding gradient goes through shared memory to the tile scatter.
+// The multiply-adds (28 k per sample: 3.6 ms for 4.87 M samples at the FP32 cores' rate)
+// and the shared-memory loads that feed them bound it.  One thread per sample with 128
+// threads per SM, whose weight-gradient products took 8 4-byte loads for 16 multiply-adds,
+// needed 14.2 ms there; this form 7.9 ms (8.6 with 2 samples x 16 outputs per thread).
 constexpr int kTile = 128;
-constexpr int kRow = 261;  // per-sample activation row (odd stride: conflict-free per-thread access)
-// Row layout: f[0,32) h1[32,96) x3[96,128) h3[128,192) h4[192,256) dz[256,259)
-constexpr int kRf = 0, kRh1 = 32, kRx3 = 96, kRh3 = 128, kRh4 = 192, kRdz = 256;
+constexpr int kBwdThreadsF = 256;
+constexpr int kRow = 260;  // 16-byte rows; consecutive rows start 16 bytes apart modulo the banks
+// Row layout: f[0,32) h1[32,96) x3[96,128) h3[128,192) h4[192,256), then the colour
+// seeds (dL/dc, later dL/dz) and dL/dsigma (later dL/dsigma * dsigma/dh_0)
+constexpr int kRf = 0, kRh1 = 32, kRx3 = 96, kRh3 = 128, kRh4 = 192, kRdz = 256, kRds = 259;
 
 struct SmemBwd {
     float W[kMlpParams];          // plain (out, in) layout as in the parameter buffer
-    float dW[kMlpParams];         // gradient accumulators
-    float act[kTile * kRow];
+    float act[kTile * kRow];      // at the end: the block's weight gradients
+    float2 df[kTile * 16];        // dL/dfeat by tile_df
+    float4 pos[2][kTile];         // sample positions by tile_row, by tile parity
 };
+static_assert(kMlpParams % 4 == 0, "rows of 16 bytes behind the weights");
 
-// dW[n][k] += sum_s A[s][a_off + n] * B[s][b_off + k] for an (NO x NI) weight,
-// 4x4 register blocks distributed over the block's threads.
-__device__ __forceinline__ void tile_outer(const float* __restrict__ act, int a_off, int b_off,
-                                           int NO, int NI, float* __restrict__ dW) {
-    const int nb_i = NI / 4;
-    const int n_blocks = (NO / 4) * nb_i;
-    for (int blk = threadIdx.x; blk < n_blocks; blk += blockDim.x) {
-        const int n0 = (blk / nb_i) * 4, k0 = (blk % nb_i) * 4;
-        float acc[4][4] = {};
-        for (int sidx = 0; sidx < kTile; ++sidx) {
-            const float* row = act + sidx * kRow;
-            float a[4], b[4];
+// o[n][q] += sum_k W[n][k] x_q[k] for NO outputs and 4 samples (rows x, x + 32 rows, ...)
+// over K inputs, k ascending.
+template <int K, int NO>
+__device__ __forceinline__ void dot_rows(const float* __restrict__ W, const float* x, float (*o)[4]) {
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+        float4 v[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                a[q] = row[a_off + n0 + q];
-                b[q] = row[b_off + k0 + q];
-            }
+        for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const float4*>(x + 32 * q * kRow + k);
 #pragma unroll
-            for (int p = 0; p < 4; ++p)
+        for (int n = 0; n < NO; ++n) {
+            const float4 w = *reinterpret_cast<const float4*>(W + n * K + k);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] += a[p] * b[q];
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.x, v[q].x, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.y, v[q].y, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.z, v[q].z, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.w, v[q].w, o[n][q]);
+        }
+    }
+}
+
+// o[k][q] += sum_n W[n][k] g_q[n] for NO consecutive k over N rows of length LD.
+template <int N, int LD, int NO>
+__device__ __forceinline__ void dot_cols(const float* __restrict__ W, const float* g, float (*o)[4]) {
+#pragma unroll 1
+    for (int n = 0; n < N; n += 4) {
+        float v[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 t = *reinterpret_cast<const float4*>(g + 32 * q * kRow + n);
+            v[0][q] = t.x;
+            v[1][q] = t.y;
+            v[2][q] = t.z;
+            v[3][q] = t.w;
         }
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
+        for (int i = 0; i < 4; ++i) {
+            float w[NO];
+            if constexpr (NO % 4 == 0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) dW[(n0 + p) * NI + k0 + q] += acc[p][q];
+                for (int k = 0; k < NO; k += 4) {
+                    const float4 t = *reinterpret_cast<const float4*>(W + (n + i) * LD + k);
+                    w[k] = t.x;
+                    w[k + 1] = t.y;
+                    w[k + 2] = t.z;
+                    w[k + 3] = t.w;
+                }
+            } else {
+                const float2 t = *reinterpret_cast<const float2*>(W + (n + i) * LD);
+                w[0] = t.x;
+                w[1] = t.y;
+            }
+#pragma unroll
+            for (int k = 0; k < NO; ++k)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) o[k][q] = fmaf(w[k], v[i][q], o[k][q]);
+        }
     }
+}
+
+// acc[4 n + j] += sum_s g[s][n] x[s][j] over samples s0 .. s0 + ns - 1, 8 rows n and 4
+// columns j (g, x: the thread's first row and column in the activation rows).
+__device__ __forceinline__ void outer_sum(const float* g, const float* x, int s0, int ns, float* acc) {
+    g += s0 * kRow;
+    x += s0 * kRow;
+#pragma unroll 2
+    for (int s = 0; s < ns; ++s, g += kRow, x += kRow) {
+        const float4 xv = *reinterpret_cast<const float4*>(x);
+#pragma unroll
+        for (int n = 0; n < 8; n += 4) {
+            const float4 gv = *reinterpret_cast<const float4*>(g + n);
+            const float gn[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                acc[4 * (n + m)] = fmaf(gn[m], xv.x, acc[4 * (n + m)]);
+                acc[4 * (n + m) + 1] = fmaf(gn[m], xv.y, acc[4 * (n + m) + 1]);
+                acc[4 * (n + m) + 2] = fmaf(gn[m], xv.z, acc[4 * (n + m) + 2]);
+                acc[4 * (n + m) + 3] = fmaf(gn[m], xv.w, acc[4 * (n + m) + 3]);
+            }
+        }
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void zero(float* v) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = 0.f;
+}
+
+// Output n of sample q, N of them (a multiple of 4, or 2), to the samples' rows.
+template <int N, bool RELU>
+__device__ __forceinline__ void put(float* dst, const float (*o)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) v[n] = RELU ? fmaxf(o[n][q], 0.f) : o[n][q];
+        float* d = dst + 32 * q * kRow;
+        if constexpr (N % 4 == 0) {
+#pragma unroll
+            for (int n = 0; n < N; n += 4)
+                *reinterpret_cast<float4*>(d + n) = make_float4(v[n], v[n + 1], v[n + 2], v[n + 3]);
+        } else {
+            *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
+        }
+    }
+}
+
+// 8 gradients of 4 samples over their activations (masked by the ReLU branches those tell).
+__device__ __forceinline__ void put_masked(float* act, const float (*o)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int n = 0; n < 8; n += 4) {
+            float4* a = reinterpret_cast<float4*>(act + 32 * q * kRow + n);
+            const float4 h = *a;
+            *a = make_float4(h.x > 0.f ? o[n][q] : 0.f, h.y > 0.f ? o[n + 1][q] : 0.f,
+                             h.z > 0.f ? o[n + 2][q] : 0.f, h.w > 0.f ? o[n + 3][q] : 0.f);
+        }
 }
 
 // kPose: also writes, per sample, dL/dp (world position) and the view-direction
 // gradient through the SH encoding into pose_s[2 i], pose_s[2 i + 1].
 template <bool kPose>
-__global__ void __launch_bounds__(kTile) k_field_bwd_fp32(DevCfg c, const float* __restrict__ params,
+__global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const float* __restrict__ params,
                                                           float* __restrict__ grads,
                                                           const float* __restrict__ rays, uint32_t cap,
                                                           const uint32_t* __restrict__ n_total,
@@ -194,205 +305,220 @@ __global__ void __launch_bounds__(kTile) k_field_bwd_fp32(DevCfg c, const float*
                                                           const float* __restrict__ feat,
                                                           const float4* __restrict__ dsig_rgb,
                                                           float4* __restrict__ pose_s) {
-    extern __shared__ float smem_raw[];
+    extern __shared__ __align__(16) float smem_raw[];
     SmemBwd& s = *reinterpret_cast<SmemBwd*>(smem_raw);
+    const uint32_t n = *n_total;
+    if (blockIdx.x * (uint32_t)kTile >= n) return;
     const float* mlp = params + (size_t)c.L * c.T * 2;
-    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) {
-        s.W[i] = mlp[i];
-        s.dW[i] = 0.f;
-    }
-    __syncthreads();
+    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) s.W[i] = mlp[i];
     const float* W1 = s.W + kOffW1;
     const float* W2 = s.W + kOffW2;
     const float* W3 = s.W + kOffW3;
     const float* W4 = s.W + kOffW4;
     const float* W5 = s.W + kOffW5;
-    const uint32_t n = *n_total;
     float2* gtables = reinterpret_cast<float2*>(grads);
-    float* row = s.act + threadIdx.x * kRow;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // layer products: samples lane, lane + 32, ..., the warp's eighth of the outputs
+    float* const row0 = s.act + lane * kRow;
+    // weight gradients: 4 columns and 8 rows per thread.  64 columns are 16 lanes (a half
+    // warp each other samples or rows), 32 columns 8 lanes.
+    const int c16 = 4 * (lane & 15), c8 = 4 * (lane & 7), half = lane >> 4, quart = lane >> 3, e0 = warp * 16;
+    const uint32_t level = scatter_level(c, tid);
+    float g1[32], g2[32], g3[32], g4[32], g5[6];
+    zero<32>(g1);
+    zero<32>(g2);
+    zero<32>(g3);
+    zero<32>(g4);
+    zero<6>(g5);
     const uint32_t n_tiles = (n + kTile - 1) / kTile;
-    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const uint32_t i = tile * kTile + threadIdx.x;
-        const bool valid = i < n;
-        float3 x = make_float3(0.f, 0.f, 0.f);
-        float3 d = make_float3(0.f, 0.f, 0.f);
-        float dsig = 0.f, sigma = 0.f;
-        bool sig_grad_off = false;
-        if (valid) {
-            // ---- recompute the forward pass into this sample's row
-            x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
-            float f[kEnc];
-            const float4* fi = reinterpret_cast<const float4*>(feat + (size_t)i * kEnc);
+    uint32_t parity = 0;
+    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, parity ^= 1u) {
+        const uint32_t i0 = tile * kTile;
+        {   // inputs: two threads per sample
+            const int r = tid & 127, part = tid >> 7;
+            const uint32_t i = i0 + r;
+            const bool valid = i < n;
+            float* row = s.act + r * kRow;
+            float4 v[4];
+            const float4* fi = reinterpret_cast<const float4*>(feat + (size_t)i * kEnc) + 4 * part;
 #pragma unroll
-            for (int k = 0; k < kEnc / 4; ++k) {
-                const float4 v = fi[k];
-                f[4 * k] = v.x; f[4 * k + 1] = v.y; f[4 * k + 2] = v.z; f[4 * k + 3] = v.w;
-            }
-#pragma unroll
-            for (int k = 0; k < kEnc; ++k) row[kRf + k] = f[k];
-            float y[kGeo];
-#pragma unroll
-            for (int m = 0; m < kGeo; ++m) y[m] = 0.f;
-#pragma unroll 2
-            for (int j = 0; j < kHid; ++j) {
-                float a = 0.f;
-#pragma unroll
-                for (int k = 0; k < kEnc; ++k) a += W1[j * kEnc + k] * f[k];
-                a = fmaxf(a, 0.f);
-                row[kRh1 + j] = a;
-#pragma unroll
-                for (int m = 0; m < kGeo; ++m) y[m] += W2[m * kHid + j] * a;
-            }
-            float x3[32];
-#pragma unroll
-            for (int m = 0; m < kGeo; ++m) x3[m] = y[m];
-            sh16(d.x, d.y, d.z, x3 + kGeo);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) row[kRx3 + k] = x3[k];
-            sigma = expf(fminf(x3[0], kSigmaHMax));
-            if (!(x3[0] < kSigmaHMax)) sig_grad_off = true;
-            float h4[kHid];
-#pragma unroll
-            for (int q = 0; q < kHid; ++q) h4[q] = 0.f;
-#pragma unroll 1
-            for (int j = 0; j < kHid; ++j) {
-                float a = 0.f;
-#pragma unroll
-                for (int k = 0; k < 32; ++k) a += W3[j * 32 + k] * x3[k];
-                a = fmaxf(a, 0.f);
-                row[kRh3 + j] = a;
-#pragma unroll
-                for (int q = 0; q < kHid; ++q) h4[q] += W4[q * kHid + j] * a;
-            }
-            float z0 = 0.f, z1 = 0.f, z2 = 0.f;
-#pragma unroll
-            for (int q = 0; q < kHid; ++q) {
-                const float h = fmaxf(h4[q], 0.f);
-                row[kRh4 + q] = h;
-                z0 += W5[q] * h;
-                z1 += W5[kHid + q] * h;
-                z2 += W5[2 * kHid + q] * h;
-            }
-            const float4 g = dsig_rgb[i];
-            dsig = g.x;
-            const float c0 = sigmoidf_(z0), c1 = sigmoidf_(z1), c2 = sigmoidf_(z2);
-            row[kRdz + 0] = g.y * c0 * (1.f - c0);
-            row[kRdz + 1] = g.z * c1 * (1.f - c1);
-            row[kRdz + 2] = g.w * c2 * (1.f - c2);
-        } else {
-            for (int k = 0; k < kRow; ++k) row[k] = 0.f;
-        }
-        __syncthreads();
-        // dW5[c][q] += sum_s dz[s][c] h4[s][q]
-        for (int e = threadIdx.x; e < 3 * kHid; e += blockDim.x) {
-            const int cc = e / kHid, q = e % kHid;
-            float acc = 0.f;
-            for (int sidx = 0; sidx < kTile; ++sidx)
-                acc += s.act[sidx * kRow + kRdz + cc] * s.act[sidx * kRow + kRh4 + q];
-            s.dW[kOffW5 + e] += acc;
-        }
-        __syncthreads();
-        // dA4 = (W5^T dz) * [h4 > 0]  (overwrites h4)
-        {
-            const float dz0 = row[kRdz], dz1 = row[kRdz + 1], dz2 = row[kRdz + 2];
-#pragma unroll 8
-            for (int q = 0; q < kHid; ++q) {
-                const float dh = W5[q] * dz0 + W5[kHid + q] * dz1 + W5[2 * kHid + q] * dz2;
-                row[kRh4 + q] = row[kRh4 + q] > 0.f ? dh : 0.f;
-            }
-        }
-        __syncthreads();
-        tile_outer(s.act, kRh4, kRh3, kHid, kHid, s.dW + kOffW4);   // dW4 = dA4^T h3
-        __syncthreads();
-        // dA3 = (W4^T dA4) * [h3 > 0]  (overwrites h3)
-        {
-            float dh[kHid];
-#pragma unroll
-            for (int q = 0; q < kHid; ++q) dh[q] = 0.f;
-#pragma unroll 1
-            for (int nn = 0; nn < kHid; ++nn) {
-                const float a = row[kRh4 + nn];
-#pragma unroll
-                for (int q = 0; q < kHid; ++q) dh[q] += W4[nn * kHid + q] * a;
-            }
-#pragma unroll
-            for (int q = 0; q < kHid; ++q) row[kRh3 + q] = row[kRh3 + q] > 0.f ? dh[q] : 0.f;
-        }
-        __syncthreads();
-        tile_outer(s.act, kRh3, kRx3, kHid, 32, s.dW + kOffW3);     // dW3 = dA3^T x3
-        __syncthreads();
-        // dy = (W3^T dA3)[0:16], dy_0 += dL/dsigma * sigma  (overwrites x3[0:16])
-        {
-            float dy[kGeo];
-#pragma unroll
-            for (int m = 0; m < kGeo; ++m) dy[m] = 0.f;
-#pragma unroll 4
-            for (int nn = 0; nn < kHid; ++nn) {
-                const float a = row[kRh3 + nn];
-#pragma unroll
-                for (int m = 0; m < kGeo; ++m) dy[m] += W3[nn * 32 + m] * a;
-            }
-            if (!sig_grad_off) dy[0] += dsig * sigma;
-            if (kPose) {
-                // the SH inputs' gradient (W3^T dA3)[16:32] -> the view-direction gradient
-                float dsh[kSH];
-#pragma unroll
-                for (int m = 0; m < kSH; ++m) dsh[m] = 0.f;
-#pragma unroll 4
-                for (int nn = 0; nn < kHid; ++nn) {
-                    const float a = row[kRh3 + nn];
-#pragma unroll
-                    for (int m = 0; m < kSH; ++m) dsh[m] += W3[nn * 32 + kGeo + m] * a;
+            for (int k = 0; k < 4; ++k) v[k] = valid ? fi[k] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (part == 0) {
+                float3 x = make_float3(0.f, 0.f, 0.f), d = x;
+                float sh[16];
+                zero<16>(sh);
+                if (valid) {
+                    x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
+                    sh16(d.x, d.y, d.z, sh);
                 }
-                const float3 gd = sh16_vjp(d.x, d.y, d.z, dsh);
-                if (valid) pose_s[2 * (size_t)i + 1] = make_float4(gd.x, gd.y, gd.z, 0.f);
+                s.pos[parity][tile_row(r)] = make_float4(x.x, x.y, x.z, 0.f);
+                #pragma unroll
+                for (int k = 0; k < 16; k += 4)
+                    *reinterpret_cast<float4*>(row + kRx3 + kGeo + k) = make_float4(sh[k], sh[k + 1], sh[k + 2], sh[k + 3]);
+            } else {
+                const float4 g = valid ? dsig_rgb[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+                *reinterpret_cast<float4*>(row + kRdz) = make_float4(g.y, g.z, g.w, g.x);
             }
 #pragma unroll
-            for (int m = 0; m < kGeo; ++m) row[kRx3 + m] = dy[m];
+            for (int k = 0; k < 4; ++k) *reinterpret_cast<float4*>(row + kRf + 16 * part + 4 * k) = v[k];
         }
         __syncthreads();
-        tile_outer(s.act, kRx3, kRh1, kGeo, kHid, s.dW + kOffW2);   // dW2 = dy^T h1
+        float o[8][4];
+        // ---- forward recompute
+        zero<32>(&o[0][0]);
+        dot_rows<kEnc, 8>(W1 + 8 * warp * kEnc, row0 + kRf, o);
+        put<8, true>(row0 + kRh1 + 8 * warp, o);
         __syncthreads();
-        // dA1 = (W2^T dy) * [h1 > 0]  (overwrites h1)
-        {
-            float dy[kGeo];
-#pragma unroll
-            for (int m = 0; m < kGeo; ++m) dy[m] = row[kRx3 + m];
+        zero<8>(&o[0][0]);
+        dot_rows<kHid, 2>(W2 + 2 * warp * kHid, row0 + kRh1, o);
+        put<2, false>(row0 + kRx3 + 2 * warp, o);
+        __syncthreads();
+        zero<32>(&o[0][0]);
+        dot_rows<32, 8>(W3 + 8 * warp * 32, row0 + kRx3, o);
+        put<8, true>(row0 + kRh3 + 8 * warp, o);
+        __syncthreads();
+        zero<32>(&o[0][0]);
+        dot_rows<kHid, 8>(W4 + 8 * warp * kHid, row0 + kRh3, o);
+        put<8, true>(row0 + kRh4 + 8 * warp, o);
+        __syncthreads();
+        if (tid < kTile) {  // colours: dL/dz; the density's seed
+            float* row = s.act + tid * kRow;
+            float z[3] = {0.f, 0.f, 0.f};
 #pragma unroll 4
-            for (int j = 0; j < kHid; ++j) {
-                float a = 0.f;
+            for (int q = 0; q < kHid; ++q) {
+                const float h = row[kRh4 + q];
 #pragma unroll
-                for (int m = 0; m < kGeo; ++m) a += W2[m * kHid + j] * dy[m];
-                row[kRh1 + j] = row[kRh1 + j] > 0.f ? a : 0.f;
+                for (int k = 0; k < 3; ++k) z[k] = fmaf(W5[k * kHid + q], h, z[k]);
             }
+            float4 g = *reinterpret_cast<const float4*>(row + kRdz);
+            const float c0 = sigmoidf_(z[0]), c1 = sigmoidf_(z[1]), c2 = sigmoidf_(z[2]);
+            const float y0 = row[kRx3];
+            g.x = g.x * c0 * (1.f - c0);
+            g.y = g.y * c1 * (1.f - c1);
+            g.z = g.z * c2 * (1.f - c2);
+            g.w = y0 < kSigmaHMax ? g.w * expf(fminf(y0, kSigmaHMax)) : 0.f;
+            *reinterpret_cast<float4*>(row + kRdz) = g;
         }
         __syncthreads();
-        tile_outer(s.act, kRh1, kRf, kHid, kEnc, s.dW + kOffW1);    // dW1 = dA1^T f
-        // df = W1^T dA1, scattered into the tables (all lanes take part)
-        {
+        // ---- backward.  dW5 += dz^T h4
+#pragma unroll 4
+        for (int q = e0; q < e0 + 16; ++q) {
+            const float4 g = *reinterpret_cast<const float4*>(s.act + q * kRow + kRdz);
+            const float2 h = *reinterpret_cast<const float2*>(s.act + q * kRow + kRh4 + 2 * lane);
+            g5[0] = fmaf(g.x, h.x, g5[0]);
+            g5[1] = fmaf(g.x, h.y, g5[1]);
+            g5[2] = fmaf(g.y, h.x, g5[2]);
+            g5[3] = fmaf(g.y, h.y, g5[3]);
+            g5[4] = fmaf(g.z, h.x, g5[4]);
+            g5[5] = fmaf(g.z, h.y, g5[5]);
+        }
+        // dA4 = (W5^T dz) [h4 > 0]
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 p = *reinterpret_cast<const float4*>(row0 + 32 * q * kRow + kRdz);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                o[k][q] = W5[8 * warp + k] * p.x + W5[kHid + 8 * warp + k] * p.y + W5[2 * kHid + 8 * warp + k] * p.z;
+        }
+        __syncthreads();
+        put_masked(row0 + kRh4 + 8 * warp, o);
+        __syncthreads();
+        // dW4 += dA4^T h3;  dA3 = (W4^T dA4) [h3 > 0]
+        outer_sum(s.act + kRh4 + 8 * warp, s.act + kRh3 + c16, 64 * half, 64, g4);
+        zero<32>(&o[0][0]);
+        dot_cols<kHid, kHid, 8>(W4 + 8 * warp, row0 + kRh4, o);
+        __syncthreads();
+        put_masked(row0 + kRh3 + 8 * warp, o);
+        __syncthreads();
+        // dW3 += dA3^T x3;  dy = (W3^T dA3)[0:16], dy_0 += the density's seed
+        outer_sum(s.act + kRh3 + 8 * warp, s.act + kRx3 + c8, 32 * quart, 32, g3);
+        if (kPose && tid < kTile && i0 + tid < n) {
+            // the SH inputs' gradient (W3^T dA3)[16:32] -> the view-direction gradient
+            const float* row = s.act + tid * kRow;
+            float dsh[kSH];
+            zero<kSH>(dsh);
+#pragma unroll 4
+            for (int nn = 0; nn < kHid; ++nn) {
+                const float gg = row[kRh3 + nn];
+#pragma unroll
+                for (int m = 0; m < kSH; ++m) dsh[m] += W3[nn * 32 + kGeo + m] * gg;
+            }
+            const uint32_t r = ray_id[i0 + tid];
+            const float3 gd = sh16_vjp(rays[kDx * cap + r], rays[kDy * cap + r], rays[kDz * cap + r], dsh);
+            pose_s[2 * (size_t)(i0 + tid) + 1] = make_float4(gd.x, gd.y, gd.z, 0.f);
+        }
+        zero<8>(&o[0][0]);
+        dot_cols<kHid, 32, 2>(W3 + 2 * warp, row0 + kRh3, o);
+        if (warp == 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[0][q] += row0[32 * q * kRow + kRds];
+        }
+        __syncthreads();
+        put<2, false>(row0 + kRx3 + 2 * warp, o);
+        __syncthreads();
+        // dW2 += dy^T h1;  dA1 = (W2^T dy) [h1 > 0]
+        outer_sum(s.act + kRx3 + 8 * half, s.act + kRh1 + c16, e0, 16, g2);
+        zero<32>(&o[0][0]);
+        dot_cols<kGeo, kHid, 8>(W2 + 8 * warp, row0 + kRx3, o);
+        __syncthreads();
+        put_masked(row0 + kRh1 + 8 * warp, o);
+        __syncthreads();
+        // dW1 += dA1^T f;  df = W1^T dA1, scattered into the tables
+        outer_sum(s.act + kRh1 + 8 * warp, s.act + kRf + c8, 32 * quart, 32, g1);
+        zero<16>(&o[0][0]);
+        dot_cols<kHid, kEnc, 4>(W1 + 4 * warp, row0 + kRh1, o);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s.df[tile_df(lane + 32 * q, 2 * warp)] = make_float2(o[0][q], o[1][q]);
+            s.df[tile_df(lane + 32 * q, 2 * warp + 1)] = make_float2(o[2][q], o[3][q]);
+        }
+        __syncthreads();
+        scatter_tile(c, gtables, tid, level, s.pos[parity], s.df, n - i0);
+        if (kPose && tid < kTile && i0 + tid < n) {
             float df[kEnc];
 #pragma unroll
-            for (int k = 0; k < kEnc; ++k) df[k] = 0.f;
-            if (valid) {
-#pragma unroll 2
-                for (int j = 0; j < kHid; ++j) {
-                    const float a = row[kRh1 + j];
-#pragma unroll
-                    for (int k = 0; k < kEnc; ++k) df[k] += W1[j * kEnc + k] * a;
-                }
+            for (int q = 0; q < 16; ++q) {
+                const float2 v = s.df[tile_df(tid, q)];
+                df[2 * q] = v.x;
+                df[2 * q + 1] = v.y;
             }
-            hash_scatter_warp(c, gtables, x, [&](int l) { return make_float2(df[2 * l], df[2 * l + 1]); },
-                                     valid);
-            if (kPose && valid) {
-                const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params), x, df);
-                pose_s[2 * (size_t)i] = make_float4(gx.x * c.inv_size, gx.y * c.inv_size, gx.z * c.inv_size, 0.f);
+            const float4 x = s.pos[parity][tile_row(tid)];
+            const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params), make_float3(x.x, x.y, x.z), df);
+            pose_s[2 * (size_t)(i0 + tid)] = make_float4(gx.x * c.inv_size, gx.y * c.inv_size, gx.z * c.inv_size, 0.f);
+        }
+        // the next tile's inputs go to rows that nobody reads any more, and to the other
+        // position buffer; dL/dfeat is written again many barriers later
+    }
+    // ---- the warps' sums meet in shared memory (act), one part after the other
+    __syncthreads();
+    float* dW = s.act;
+    for (int i = tid; i < kMlpParams; i += kBwdThreadsF) dW[i] = 0.f;
+    auto add = [&](int off, int ld, const float* g) {
+#pragma unroll
+        for (int n = 0; n < 8; ++n)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dW[off + n * ld + k] += g[4 * n + k];
+    };
+    for (int part = 0; part < 8; ++part) {
+        __syncthreads();
+        if (half == part) add(kOffW4 + 8 * warp * kHid + c16, kHid, g4);
+        if (quart == part) {
+            add(kOffW3 + 8 * warp * 32 + c8, 32, g3);
+            add(kOffW1 + 8 * warp * kEnc + c8, kEnc, g1);
+        }
+        if (warp == part) {
+            add(kOffW2 + 8 * half * kHid + c16, kHid, g2);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                dW[kOffW5 + k * kHid + 2 * lane] += g5[2 * k];
+                dW[kOffW5 + k * kHid + 2 * lane + 1] += g5[2 * k + 1];
             }
         }
-        __syncthreads();
     }
+    __syncthreads();
     float* gmlp = grads + (size_t)c.L * c.T * 2;
-    for (int e = threadIdx.x; e < kMlpParams; e += blockDim.x) {
-        const float v = s.dW[e];
+    for (int e = tid; e < kMlpParams; e += kBwdThreadsF) {
+        const float v = dW[e];
         if (v != 0.f) atomicAdd(gmlp + e, v);
     }
 }
@@ -404,12 +530,13 @@ void launch_field_bwd_fp32(const DevCfg& c, const float* params, float* grads, u
     cudaFuncSetAttribute(k_field_bwd_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_field_bwd_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (pose)
-        k_field_bwd_fp32<true><<<n_sm, kTile, smem, st>>>(c, params, grads, b.rays, b.cap_rays, b.offsets + n_rays,
-                                                          b.ray_id, b.t, b.feat, b.dsig_rgb, b.pose_s);
+        k_field_bwd_fp32<true><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
+                                                                 b.offsets + n_rays, b.ray_id, b.t, b.feat, b.dsig_rgb,
+                                                                 b.pose_s);
     else
-        k_field_bwd_fp32<false><<<n_sm, kTile, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
-                                                           b.offsets + n_rays, b.ray_id, b.t, b.feat, b.dsig_rgb,
-                                                           nullptr);
+        k_field_bwd_fp32<false><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
+                                                                  b.offsets + n_rays, b.ray_id, b.t, b.feat,
+                                                                  b.dsig_rgb, nullptr);
 }
 
 }  // namespace nm
