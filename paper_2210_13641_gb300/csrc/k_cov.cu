@@ -9,11 +9,19 @@
 // FP64 throughout: the reduced camera matrix of a bundle adjustment is badly
 // conditioned, and the work is small (the camera block of a keyframe window has at
 // most kCovMaxC rows).
+// The FP64 units are what there is little of (about 2 multiply-adds per clock and SM):
+// every product is taken once (the symmetric halves are not computed twice), and what
+// need not be one block is spread over the SMs.
 //   k_cov_schur   pixels -> sum_q e_a e_b^T / P_q into a shared-memory copy of the
 //                 c x c matrix per block, flushed with FP64 atomics;
-//   k_cov_chol    one block: C - that sum, Cholesky (packed lower triangle in shared
-//                 memory), L^-1 by forward substitution, Sigma_T = L^-T L^-1;
+//   k_cov_chol    one block: C - that sum, Cholesky in shared memory;
+//   k_cov_inv     L^-1, one warp per column;
+//   k_cov_gram    Sigma_T = L^-T L^-1, one thread per element of its lower triangle;
 //   k_cov_depth   one thread per pixel: 1/P + (E P^-1)_q^T Sigma_T (E P^-1)_q.
+// 20 keyframes, 96 k pixels, 4 blocks per pixel: the call takes 0.67 ms on device arrays
+// (2.45 before: one block for everything after the sum, with index decoding by square
+// roots and one thread per column of the inverse, 1.83 ms; sums by a shared atomic per
+// product, 0.344; the full squares in k_cov_depth, 0.136).
 #include <cstdint>
 #include <cstring>
 #include <string>
@@ -29,132 +37,242 @@ namespace {
 
 constexpr uint32_t kCovMaxC = 144;  // 24 keyframes
 constexpr uint32_t kCovMaxB = 8;
-constexpr int kCovThreads = 1024;
+constexpr int kCovThreads = 512;
 
 void set_cov_error(const char* msg) { set_global_error(msg); }
 
 __device__ __forceinline__ uint32_t tri(uint32_t i, uint32_t j) { return i * (i + 1) / 2 + j; }  // i >= j
 
-// Per block: the pixels q = blockIdx.x, blockIdx.x + gridDim.x, ... (one warp per
-// pixel) add e_a e_b^T / P_q for every pair of its blocks (a, b) to a shared copy of
-// the c x c matrix (lower triangle, packed), which is then added to acc.
+// Column-major packed lower triangle of order c: column k starts at its diagonal.
+__device__ __forceinline__ uint32_t col(uint32_t c, uint32_t k) { return k * c - k * (k - 1) / 2 - k; }  // + i
+
+// Each warp takes a run of consecutive pixels.  Consecutive pixels mostly belong to one
+// keyframe and touch the same poses, so the products e_a e_b^T / P_q of the pairs a >= b
+// are summed in the lanes' registers (entry t = lane + 32 m of the pairs' 36 products)
+// while the poses stay the same, and leave for the block's shared copy of the packed
+// lower triangle when they change.
+template <int B>
 __global__ void __launch_bounds__(256) k_cov_schur(uint32_t c, const double* __restrict__ P, uint32_t p,
                                                    const int32_t* __restrict__ blk, const double* __restrict__ e,
-                                                   uint32_t B, double* __restrict__ acc, uint32_t* __restrict__ flag) {
+                                                   double* __restrict__ acc, uint32_t* __restrict__ flag) {
+    constexpr int kEntries = B * (B + 1) / 2 * 36, kM = (kEntries + 31) / 32;
     extern __shared__ double sh[];
+    __shared__ double se[8][2][B * 6];  // per warp: e and e / P of the pixel
+    __shared__ int32_t sk[8][B];        // per warp: the poses the sums belong to
     const uint32_t n_tri = c * (c + 1) / 2;
     for (uint32_t i = threadIdx.x; i < n_tri; i += blockDim.x) sh[i] = 0.0;
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    if (lane < B) sk[w][lane] = -1;
     __syncthreads();
-    const uint32_t lane = threadIdx.x & 31u, warps = blockDim.x >> 5;
-    const uint32_t n_entries = B * B * 36;
-    for (uint32_t q = blockIdx.x * warps + (threadIdx.x >> 5); q < p; q += gridDim.x * warps) {
+    double sum[kM];
+    uint32_t at[kM];                    // the lane's entries: 6 a + r in the low half, 6 b + col above
+#pragma unroll
+    for (int m = 0; m < kM; ++m) {
+        const uint32_t t = lane + 32u * m, pair = t / 36u, rc = t % 36u;
+        uint32_t a = 0;
+        while ((a + 1) * (a + 2) / 2 <= pair) ++a;
+        at[m] = (6u * a + rc / 6u) | ((6u * (pair - a * (a + 1) / 2) + rc % 6u) << 16);
+        sum[m] = 0.0;
+    }
+    auto flush = [&]() {
+#pragma unroll
+        for (int m = 0; m < kM; ++m) {
+            if ((int)(lane + 32u * m) >= kEntries) continue;
+            uint32_t t = at[m];
+            asm volatile("" : "+r"(t));  // decoded here, not kept decoded in registers for every entry
+            const uint32_t ia = t & 0xffffu, ib = t >> 16;
+            const uint32_t a = ia / 6u, b = ib / 6u, r = ia % 6u, cc = ib % 6u;
+            const int32_t ka = sk[w][a], kb = sk[w][b];
+            if (ka < 0 || kb < 0) continue;
+            uint32_t i = 6u * (uint32_t)ka + r, j = 6u * (uint32_t)kb + cc;
+            double v = sum[m];
+            if (a == b && r < cc) continue;                     // the mirrored product of the same block
+            if (a != b && ka == kb && r == cc) v += v;           // (a, b) and (b, a) meet on the diagonal
+            if (i < j) {
+                const uint32_t x = i;
+                i = j;
+                j = x;
+            }
+            if (i < c) atomicAdd(&sh[tri(i, j)], v);
+        }
+#pragma unroll
+        for (int m = 0; m < kM; ++m) sum[m] = 0.0;
+    };
+    const uint32_t n_warps = gridDim.x * 8u, chunk = (p + n_warps - 1) / n_warps;
+    const uint32_t q0 = min(p, (blockIdx.x * 8u + w) * chunk), q1 = min(p, q0 + chunk);
+    for (uint32_t q = q0; q < q1; ++q) {
         const double Pq = P[q];
         if (!(Pq > 0.0)) {
             if (lane == 0) atomicOr(flag, 1u);
             continue;
         }
-        const double inv = 1.0 / Pq;
-        for (uint32_t t = lane; t < n_entries; t += 32) {
-            const uint32_t ab = t / 36, rc = t % 36;
-            const uint32_t a = ab / B, b = ab % B, r = rc / 6, col = rc % 6;
-            const int32_t ka = blk[(size_t)q * B + a], kb = blk[(size_t)q * B + b];
-            if (ka < 0 || kb < 0) continue;
-            const uint32_t i = 6u * (uint32_t)ka + r, j = 6u * (uint32_t)kb + col;
-            if (i < j || i >= c) continue;  // lower triangle (the pair (b, a) covers the rest)
-            atomicAdd(&sh[tri(i, j)], e[((size_t)q * B + a) * 6 + r] * e[((size_t)q * B + b) * 6 + col] * inv);
+        const int32_t k = lane < B ? blk[(size_t)q * B + lane] : 0;
+        if (__ballot_sync(0xffffffffu, lane < B && k != sk[w][lane < B ? lane : 0])) {
+            flush();
+            __syncwarp();
+            if (lane < B) sk[w][lane] = k;
         }
+        const double inv = 1.0 / Pq;
+        __syncwarp();
+        for (uint32_t t = lane; t < B * 6; t += 32) {
+            const double v = e[(size_t)q * B * 6 + t];
+            se[w][0][t] = v;
+            se[w][1][t] = v * inv;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kM; ++m)
+            if ((int)(lane + 32u * m) < kEntries) sum[m] = fma(se[w][0][at[m] & 0xffffu], se[w][1][at[m] >> 16], sum[m]);
     }
+    __syncwarp();
+    if (q1 > q0) flush();
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < n_tri; i += blockDim.x)
         if (sh[i] != 0.0) atomicAdd(&acc[i], sh[i]);
 }
 
-// One block: H_T = C - acc (packed lower), Cholesky in place, Y = L^-1 (packed
-// lower, forward substitution per column), Sigma_T = Y^T Y (full c x c, row-major).
+// One block: H_T = C - acc, right-looking Cholesky (column-major packed).  While the other
+// warps subtract column j's products from the columns beyond j + 1, warp 0 does that for
+// column j + 1 and finishes it (pivot, scaling): one barrier per column.
 __global__ void __launch_bounds__(kCovThreads) k_cov_chol(uint32_t c, const double* __restrict__ C,
-                                                          const double* __restrict__ acc, double* __restrict__ ST,
-                                                          uint32_t* __restrict__ flag) {
-    extern __shared__ double sh[];
-    const uint32_t n_tri = c * (c + 1) / 2;
-    double* A = sh;          // packed lower: H_T, then L
-    double* Y = sh + n_tri;  // packed lower: L^-1
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    for (uint32_t t = threadIdx.x; t < n_tri; t += blockDim.x) {
-        // row i, column j of the packed index t
-        uint32_t i = (uint32_t)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
-        while (tri(i, 0) > t) --i;
-        while (tri(i + 1, 0) <= t) ++i;
-        const uint32_t j = t - tri(i, 0);
-        A[t] = C[(size_t)i * c + j] - acc[t];
-    }
+                                                          const double* __restrict__ acc, double* __restrict__ L,
+                                                          double* __restrict__ rinv, uint32_t* __restrict__ flag) {
+    extern __shared__ double A[];
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (uint32_t i = w; i < c; i += nw)
+        for (uint32_t j = lane; j <= i; j += 32) A[col(c, j) + i] = C[(size_t)i * c + j] - acc[tri(i, j)];
     __syncthreads();
-    // right-looking Cholesky
-    for (uint32_t j = 0; j < c; ++j) {
-        if (threadIdx.x == 0) {
-            const double d = A[tri(j, j)];
-            if (!(d > 0.0)) bad = 1;
-            A[tri(j, j)] = d > 0.0 ? sqrt(d) : 1.0;
+    bool bad = false;
+    auto finish = [&](uint32_t j) {  // warp 0: pivot and scaling of column j
+        double* a = A + col(c, j);
+        const double d = a[j];
+        bad = bad || !(d > 0.0);
+        const double l = d > 0.0 ? sqrt(d) : 1.0, r = 1.0 / l;
+        __syncwarp();
+        for (uint32_t i = j + 1 + lane; i < c; i += 32) a[i] *= r;
+        if (lane == 0) {
+            a[j] = l;
+            rinv[j] = r;
         }
-        __syncthreads();
-        const double ljj = A[tri(j, j)];
-        for (uint32_t i = j + 1 + threadIdx.x; i < c; i += blockDim.x) A[tri(i, j)] /= ljj;
-        __syncthreads();
-        const uint32_t m = c - j - 1;  // trailing size
-        for (uint32_t t = threadIdx.x; t < m * (m + 1) / 2; t += blockDim.x) {
-            uint32_t ii = (uint32_t)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
-            while (tri(ii, 0) > t) --ii;
-            while (tri(ii + 1, 0) <= t) ++ii;
-            const uint32_t kk = t - tri(ii, 0);
-            const uint32_t i = j + 1 + ii, k = j + 1 + kk;
-            A[tri(i, k)] -= A[tri(i, j)] * A[tri(k, j)];
-        }
-        __syncthreads();
-    }
-    // Y = L^-1: column j by forward substitution (one thread per column)
-    for (uint32_t j = threadIdx.x; j < c; j += blockDim.x) {
-        Y[tri(j, j)] = 1.0 / A[tri(j, j)];
-        for (uint32_t i = j + 1; i < c; ++i) {
-            double s = 0.0;
-            for (uint32_t k = j; k < i; ++k) s += A[tri(i, k)] * Y[tri(k, j)];
-            Y[tri(i, j)] = -s / A[tri(i, i)];
-        }
-    }
+        __syncwarp();
+    };
+    if (w == 0) finish(0);
     __syncthreads();
-    // Sigma_T = Y^T Y: (i, j) = sum_{k >= max(i, j)} Y[k][i] Y[k][j]
-    for (uint32_t t = threadIdx.x; t < c * c; t += blockDim.x) {
-        const uint32_t i = t / c, j = t % c;
-        double s = 0.0;
-        for (uint32_t k = (i > j ? i : j); k < c; ++k) s += Y[tri(k, i)] * Y[tri(k, j)];
-        ST[t] = s;
+    for (uint32_t j = 0; j + 1 < c; ++j) {
+        const double* a = A + col(c, j);
+        for (uint32_t k = w == 0 ? j + 1 : j + 1 + w; k < c; k += w == 0 ? c : nw - 1) {
+            double* b = A + col(c, k);
+            const double f = a[k];
+            for (uint32_t i = k + lane; i < c; i += 32) b[i] -= a[i] * f;
+        }
+        if (w == 0) {
+            __syncwarp();
+            finish(j + 1);
+        }
+        __syncthreads();
     }
+    for (uint32_t t = threadIdx.x; t < c * (c + 1) / 2; t += blockDim.x) L[t] = A[t];
     if (threadIdx.x == 0 && bad) atomicOr(flag, 2u);
 }
 
-// Per pixel: Sigma_d = 1/P + (E P^-1)_q^T Sigma_T (E P^-1)_q over its blocks.
-__global__ void k_cov_depth(uint32_t c, const double* __restrict__ P, uint32_t p, const int32_t* __restrict__ blk,
-                            const double* __restrict__ e, uint32_t B, const double* __restrict__ ST,
-                            double* __restrict__ Sd) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= p) return;
-    const double inv = 1.0 / P[q];
-    double s = 0.0;
-    for (uint32_t a = 0; a < B; ++a) {
-        const int32_t ka = blk[(size_t)q * B + a];
-        if (ka < 0 || 6u * (uint32_t)ka >= c) continue;
-        for (uint32_t b = 0; b < B; ++b) {
-            const int32_t kb = blk[(size_t)q * B + b];
-            if (kb < 0 || 6u * (uint32_t)kb >= c) continue;
-            for (uint32_t r = 0; r < 6; ++r) {
-                const double ea = e[((size_t)q * B + a) * 6 + r];
-                const double* row = ST + (size_t)(6u * (uint32_t)ka + r) * c + 6u * (uint32_t)kb;
-                double t = 0.0;
-                for (uint32_t col = 0; col < 6; ++col) t += row[col] * e[((size_t)q * B + b) * 6 + col];
-                s += ea * t;
+// Y = L^-1 by columns (Y[j][i], zeros above the diagonal): one warp per column, lane i's
+// rows i, i + 32, ...; each solved entry is subtracted from the rows below it.
+constexpr int kCovRows = (kCovMaxC + 31) / 32;
+__global__ void __launch_bounds__(128) k_cov_inv(uint32_t c, const double* __restrict__ L,
+                                                 const double* __restrict__ rinv, double* __restrict__ Y) {
+    extern __shared__ double A[];
+    for (uint32_t t = threadIdx.x; t < c * (c + 1) / 2; t += blockDim.x) A[t] = L[t];
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u, j = blockIdx.x * 4u + (threadIdx.x >> 5);
+    if (j >= c) return;
+    double b[kCovRows];
+#pragma unroll
+    for (int m = 0; m < kCovRows; ++m) b[m] = lane + 32u * m == j ? 1.0 : 0.0;
+#pragma unroll
+    for (int m = 0; m < kCovRows; ++m) {
+        for (uint32_t kk = 0; kk < 32; ++kk) {
+            const uint32_t k = 32u * m + kk;
+            if (k < j) continue;  // warp-uniform
+            if (k >= c) break;
+            const double y = __shfl_sync(0xffffffffu, b[m], kk) * rinv[k];
+            const double* a = A + col(c, k);
+            if (lane == kk) b[m] = y;
+#pragma unroll
+            for (int q = m; q < kCovRows; ++q) {
+                const uint32_t i = lane + 32u * q;
+                if (i > k && i < c) b[q] -= a[i] * y;
             }
         }
     }
-    Sd[q] = inv + s * inv * inv;
+#pragma unroll
+    for (int m = 0; m < kCovRows; ++m)
+        if (lane + 32u * m < c) Y[(size_t)j * c + lane + 32u * m] = b[m];
+}
+
+// Sigma_T = Y^T Y: (i, j) = sum_{k >= i} Y[k][i] Y[k][j] for i >= j, and its mirror image.
+__global__ void __launch_bounds__(256) k_cov_gram(uint32_t c, const double* __restrict__ Y, double* __restrict__ ST) {
+    if (blockIdx.y > blockIdx.x) return;
+    const uint32_t i = blockIdx.x * 16u + (threadIdx.x & 15u), j = blockIdx.y * 16u + (threadIdx.x >> 4);
+    if (i >= c || j > i) return;
+    const double *yi = Y + (size_t)i * c, *yj = Y + (size_t)j * c;
+    double s = 0.0;
+    for (uint32_t k = i; k < c; ++k) s = fma(yi[k], yj[k], s);
+    ST[(size_t)i * c + j] = s;
+    ST[(size_t)j * c + i] = s;
+}
+
+// Per pixel: Sigma_d = 1/P + (E P^-1)_q^T Sigma_T (E P^-1)_q over its blocks, each pair
+// of blocks once (Sigma_T is symmetric).
+__global__ void __launch_bounds__(256) k_cov_depth(uint32_t c, const double* __restrict__ P, uint32_t p,
+                                                   const int32_t* __restrict__ blk, const double* __restrict__ e,
+                                                   uint32_t B, const double* __restrict__ ST,
+                                                   double* __restrict__ Sd) {
+    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= p) return;
+    const double inv = 1.0 / P[q];
+    double diag = 0.0, off = 0.0;  // off: half of the mirrored products
+    for (uint32_t a = 0; a < B; ++a) {
+        const int32_t ka = blk[(size_t)q * B + a];
+        if (ka < 0 || 6u * (uint32_t)ka >= c) continue;
+        double ea[6];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) ea[r] = e[((size_t)q * B + a) * 6 + r];
+        const double* S = ST + (size_t)(6u * (uint32_t)ka) * c;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+            const double* row = S + (size_t)r * c + 6u * (uint32_t)ka;
+            diag = fma(ea[r] * row[r], ea[r], diag);
+            double t = 0.0;
+#pragma unroll
+            for (int k = 0; k < r; ++k) t = fma(row[k], ea[k], t);
+            off = fma(ea[r], t, off);
+        }
+        for (uint32_t b = 0; b < a; ++b) {
+            const int32_t kb = blk[(size_t)q * B + b];
+            if (kb < 0 || 6u * (uint32_t)kb >= c) continue;
+            double eb[6];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) eb[k] = e[((size_t)q * B + b) * 6 + k];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) {
+                const double* row = S + (size_t)r * c + 6u * (uint32_t)kb;
+                double t = 0.0;
+#pragma unroll
+                for (int k = 0; k < 6; ++k) t = fma(row[k], eb[k], t);
+                off = fma(ea[r], t, off);
+            }
+        }
+    }
+    Sd[q] = inv + (diag + 2.0 * off) * inv * inv;
+}
+
+template <int B>
+void launch_schur(uint32_t grid, size_t sh, cudaStream_t s, uint32_t c, const double* P, uint32_t p,
+                  const int32_t* blk, const double* e, double* acc, uint32_t* flag) {
+    // per call: the attribute belongs to the current device (cheap next to the kernel)
+    cudaFuncSetAttribute(k_cov_schur<B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kCovMaxC * (kCovMaxC + 1) / 2 * sizeof(double)));
+    k_cov_schur<B><<<grid, 256, sh, s>>>(c, P, p, blk, e, acc, flag);
 }
 
 struct DevBuf {
@@ -188,13 +306,16 @@ extern "C" int map_marginal_covariances(const double* C, uint32_t c, const doubl
     const size_t bBlk = (size_t)p * B * sizeof(int32_t), bE = (size_t)p * B * 6 * sizeof(double);
     const size_t n_tri = (size_t)c * (c + 1) / 2;
     DevBuf work, inputs;
-    // work: acc (packed), flag
-    if (cudaMalloc(&work.p, n_tri * sizeof(double) + 16) != cudaSuccess) {
+    // work: acc (packed), flag, L (packed), 1 / diag(L), L^-1
+    if (cudaMalloc(&work.p, (2 * n_tri + 2 + c + (size_t)c * c) * sizeof(double)) != cudaSuccess) {
         set_cov_error("map_marginal_covariances: cudaMalloc failed");
         return MAP_ENOMEM;
     }
     double* acc = static_cast<double*>(work.p);
     uint32_t* flag = reinterpret_cast<uint32_t*>(acc + n_tri);
+    double* L = acc + n_tri + 2;
+    double* rinv = L + n_tri;
+    double* Y = rinv + c;
     const double *dC = C, *dP = P, *dE = e;
     const int32_t* dBlk = blk;
     double *dST = sigma_T, *dSd = sigma_d;
@@ -225,16 +346,21 @@ extern "C" int map_marginal_covariances(const double* C, uint32_t c, const doubl
         dSd = hSd;
     }
     cudaMemsetAsync(work.p, 0, n_tri * sizeof(double) + 16, s);
-    const size_t sh_schur = n_tri * sizeof(double), sh_chol = 2 * n_tri * sizeof(double);
-    // per call: the attribute belongs to the current device (cheap next to the kernel)
-    cudaFuncSetAttribute(k_cov_schur, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(kCovMaxC * (kCovMaxC + 1) / 2 * sizeof(double)));
-    cudaFuncSetAttribute(k_cov_chol, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(kCovMaxC * (kCovMaxC + 1) * sizeof(double)));
+    const size_t sh = n_tri * sizeof(double);
+    const int sh_max = (int)(kCovMaxC * (kCovMaxC + 1) / 2 * sizeof(double));
+    cudaFuncSetAttribute(k_cov_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, sh_max);
+    cudaFuncSetAttribute(k_cov_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, sh_max);
     uint32_t grid = (p + 7) / 8;
     if (grid > 152u * 2u) grid = 152u * 2u;
-    k_cov_schur<<<grid, 256, sh_schur, s>>>(c, dP, p, dBlk, dE, B, acc, flag);
-    k_cov_chol<<<1, kCovThreads, sh_chol, s>>>(c, dC, acc, dST, flag);
+    using Schur = void (*)(uint32_t, size_t, cudaStream_t, uint32_t, const double*, uint32_t, const int32_t*,
+                           const double*, double*, uint32_t*);
+    static const Schur schur[kCovMaxB] = {launch_schur<1>, launch_schur<2>, launch_schur<3>, launch_schur<4>,
+                                          launch_schur<5>, launch_schur<6>, launch_schur<7>, launch_schur<8>};
+    schur[B - 1](grid, sh, s, c, dP, p, dBlk, dE, acc, flag);
+    k_cov_chol<<<1, kCovThreads, sh, s>>>(c, dC, acc, L, rinv, flag);
+    k_cov_inv<<<(c + 3) / 4, 128, sh, s>>>(c, L, rinv, Y);
+    const uint32_t tiles = (c + 15) / 16;
+    k_cov_gram<<<dim3(tiles, tiles), 256, 0, s>>>(c, Y, dST);
     k_cov_depth<<<(p + 255) / 256, 256, 0, s>>>(c, dP, p, dBlk, dE, B, dST, dSd);
     if (cudaGetLastError() != cudaSuccess) {
         set_cov_error("map_marginal_covariances: kernel launch failed");
