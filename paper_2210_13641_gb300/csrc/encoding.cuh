@@ -13,63 +13,68 @@ __device__ __forceinline__ float corner_weight(int k, float wx, float wy, float 
     return ((k & 1) ? wx : 1.f - wx) * ((k & 2) ? wy : 1.f - wy) * ((k & 4) ? wz : 1.f - wz);
 }
 
-// Corners k and k + 1 (k even) differ only in x.  Their slots s and s' share one
-// aligned 16-byte chunk (two float2 entries) exactly when s' = s ^ 1: in a hashed
-// level that holds whenever cx is even (the x coordinate enters the hash by xor with
-// prime 1), in a dense level whenever s is even.  The encoding reads such a pair
-// with one 16-byte load.
-__device__ __forceinline__ bool x_pair_shared(uint32_t s0, uint32_t s1) { return (s0 ^ s1) == 1u; }
+// The sample of a warp's 32 that lane `lane` encodes: lanes 2 i and 2 i + 1 have samples i
+// and 16 + i (encode_level's loads then cover 16 consecutive samples each).
+__device__ __forceinline__ uint32_t pair_sample(uint32_t lane) { return (lane >> 1) + 16u * (lane & 1u); }
 
-// Features of levels l0 .. l0 + kGatherGroup - 1 of grid position x into
-// f[0 .. 2 kGatherGroup) (zero for levels >= L).  tables: [L][T] float2.  Level by
-// level, the level's 4 x-pair loads are issued before any is used.  An x-pair of
-// corners in one chunk is read with one 16-byte load (halves swapped when corner k is
-// the upper one), any other pair with two 8-byte loads.  (Issuing the loads of 4 or 2
-// levels before using any kept more loads in flight but spilled registers in the
-// tensor-core forward: 3.18 and 3.08 ms against 3.03 ms for one level at a time.)
-constexpr int kGatherGroup = 4;
-
+// Features of level l of grid position x into f[0], f[1]; called by all 32 lanes, whose
+// positions follow pair_sample.  tables: [L][T] float2.  The gathers are bound by the
+// 128-byte lines their instructions touch in the L1 (39.5 wavefronts per sample at 73 % of
+// the data pipe when every lane read its own corners, odd x pairs in two instructions).
+// Corners k and k + 1 (k even) differ only in x and share a line 15 times in 16, so one
+// instruction reads both: the even lane the lower corner of its own sample and, in a second
+// instruction, the upper one of its neighbour's; the odd lane likewise.  Each then gets
+// its upper corner by a shuffle.  That is 27.7 lines per sample on the room workload's
+// rays instead of 43.7 (counted on the host); forward of 19.5 M samples 3.36 ms,
+// 3.66 before.  The corners are summed in the order k = 0 .. 7.
 __device__ __forceinline__ void encode_level(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
                                              float* f) {
-    const uint32_t Tmask = c.T - 1;
-    float4 q[4];   // (corner 2j, corner 2j + 1), halves swapped if bit j of swp
-    uint32_t swp = 0u;
-    float w[3];
-    const uint32_t N = c.res[l];
+    const uint32_t N = c.res[l], Tmask = c.T - 1;
     const bool dense = (c.dense_mask >> l) & 1u;
+    const bool odd = threadIdx.x & 1u;
+    const uint32_t m1 = dense ? N + 1u : 2654435761u, m2 = dense ? (N + 1u) * (N + 1u) : 805459861u;
     uint32_t cx, cy, cz;
-    level_cell(x.x, N, cx, w[0]);
-    level_cell(x.y, N, cy, w[1]);
-    level_cell(x.z, N, cz, w[2]);
+    float wx, wy, wz;
+    level_cell(x.x, N, cx, wx);
+    level_cell(x.y, N, cy, wy);
+    level_cell(x.z, N, cz, wz);
+    const uint32_t ya = cy * m1, za = cz * m2;
+    const uint32_t xn = __shfl_xor_sync(0xffffffffu, cx, 1), yn = __shfl_xor_sync(0xffffffffu, ya, 1),
+                   zn = __shfl_xor_sync(0xffffffffu, za, 1);
+    // instruction 0: the even lane's sample, 1: the odd lane's
+    const uint32_t X[2] = {odd ? xn + 1u : cx, odd ? cx : xn + 1u};
+    const uint32_t Y[2] = {odd ? yn : ya, odd ? ya : yn}, Z[2] = {odd ? zn : za, odd ? za : zn};
     const float2* tab = tables + (size_t)l * c.T;
+    float2 v[2][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint32_t yy = cy + (j & 1), zz = cz + (j >> 1);
-        const uint32_t s0 = vertex_slot(cx, yy, zz, N, dense, Tmask);
-        const uint32_t s1 = vertex_slot(cx + 1, yy, zz, N, dense, Tmask);
-        if (x_pair_shared(s0, s1)) {
-            q[j] = __ldg(reinterpret_cast<const float4*>(tab + (s0 & ~1u)));
-            swp |= (s0 & 1u) << j;
-        } else {
-            const float2 a = __ldg(tab + s0), b = __ldg(tab + s1);
-            q[j] = make_float4(a.x, a.y, b.x, b.y);
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t a = Y[i] + (j & 1) * m1, b = Z[i] + (j >> 1) * m2;
+            const uint32_t s = dense ? X[i] + a + b : (X[i] ^ a ^ b) & Tmask;
+            v[i][j] = __ldg(tab + s);
         }
     }
     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const bool hi = (swp >> j) & 1u;
-        const float4 v = q[j];
-        const float w0 = corner_weight(2 * j, w[0], w[1], w[2]);
-        const float w1 = corner_weight(2 * j + 1, w[0], w[1], w[2]);
-        a0 += w0 * (hi ? v.z : v.x);
-        a1 += w0 * (hi ? v.w : v.y);
-        a0 += w1 * (hi ? v.x : v.z);
-        a1 += w1 * (hi ? v.y : v.w);
+        const float2 lo = odd ? v[1][j] : v[0][j], snd = odd ? v[0][j] : v[1][j];
+        const float ux = __shfl_xor_sync(0xffffffffu, snd.x, 1), uy = __shfl_xor_sync(0xffffffffu, snd.y, 1);
+        const float w0 = corner_weight(2 * j, wx, wy, wz);
+        const float w1 = corner_weight(2 * j + 1, wx, wy, wz);
+        a0 += w0 * lo.x;
+        a1 += w0 * lo.y;
+        a0 += w1 * ux;
+        a1 += w1 * uy;
     }
     f[0] = a0;
     f[1] = a1;
 }
+
+// Features of levels l0 .. l0 + kGatherGroup - 1 into f[0 .. 2 kGatherGroup) (zero for
+// levels >= L), one level after the other: loads of 4 or 2 levels in flight spilled
+// registers in the tensor-core forward (3.18 and 3.08 ms against 3.03).
+constexpr int kGatherGroup = 4;
 
 __device__ __forceinline__ void encode_group(const DevCfg& c, const float2* __restrict__ tables, float3 x,
                                              int l0, float* f) {

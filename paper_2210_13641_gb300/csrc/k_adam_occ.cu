@@ -82,7 +82,8 @@ __global__ void __launch_bounds__(256) k_occ_refresh(DevCfg c, const float* __re
     const uint32_t n = R * R * R;
     const float2* tables = reinterpret_cast<const float2*>(params);
     for (uint32_t base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
-        const uint32_t cell = base + threadIdx.x;  // n is a multiple of 512: no tail
+        const uint32_t lane = threadIdx.x & 31u;
+        const uint32_t cell = base + (threadIdx.x & ~31u) + pair_sample(lane);  // n is a multiple of 512: no tail
         const uint64_t r = counter_rand(seed, kOccStream + refresh_idx, cell, 0);
         const float ux = (float)(r & 0x1FFFFFu) * (1.f / 2097152.f);
         const float uy = (float)((r >> 21) & 0x1FFFFFu) * (1.f / 2097152.f);
@@ -105,8 +106,10 @@ __global__ void __launch_bounds__(256) k_occ_refresh(DevCfg c, const float* __re
         const float sigma = expf(fminf(h0, kSigmaHMax));
         const float d = fmaxf(decay * density[cell], sigma);
         density[cell] = d;
-        const uint32_t word = __ballot_sync(0xffffffffu, d > thresh);
-        if ((threadIdx.x & 31) == 0) bits[cell >> 5] = word;
+        // bit k of the word is cell k of the warp's 32, which lane 2 k (k < 16) or 2 k - 31 has
+        const int set = __shfl_sync(0xffffffffu, (int)(d > thresh), ((lane & 15u) << 1) | (lane >> 4));
+        const uint32_t word = __ballot_sync(0xffffffffu, set);
+        if (lane == 0) bits[cell >> 5] = word;
     }
 }
 

@@ -97,13 +97,16 @@ __global__ void __launch_bounds__(128) k_field_fwd_fp32(DevCfg c, const float* _
     __syncthreads();
     const uint32_t n = *n_total;
     const float2* tables = reinterpret_cast<const float2*>(params);
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        const uint32_t i = kSel ? sel[j] : j;
-        const uint32_t r = ray_id[i];
-        float3 d;
-        const float3 x = sample_pos(c, rays, cap, r, ts[i], d);
+    for (uint32_t j0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n; j0 += gridDim.x * blockDim.x) {
+        // whole warps encode: lanes past the end stand at position 0
+        const uint32_t j = j0 + pair_sample(threadIdx.x & 31u);
+        const bool valid = j < n;
+        const uint32_t i = valid ? (kSel ? sel[j] : j) : 0u;
+        float3 d = make_float3(0.f, 0.f, 0.f), x = d;
+        if (valid) x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
         float f[kEnc];
         hash_encode(c, tables, x, f);
+        if (!valid) continue;
         if (!kSel && feat_out) {
             float4* fo = reinterpret_cast<float4*>(feat_out + (size_t)i * kEnc);
 #pragma unroll

@@ -216,7 +216,7 @@ constexpr int kFwdSmem = kWB + kT32 + kT64;                            // 45056
 
 // ------------------------------------------------------------------ forward
 // One tile of the forward: samples i0 .. min(i0 + 128, i_end) - 1; thread r of the
-// block owns sample row r.  smem: the weight tiles, then tA (128 x 32: X0, X3) and
+// block owns sample row r, the samples of a warp in pair_sample order.  smem: the weight tiles, then tA (128 x 32: X0, X3) and
 // tB (128 x 64: H1, H3, H4; a layer's MMAs have completed before its output
 // overwrites its input).  Returns after the tile's last MMA wait.
 // kSel: row r evaluates sample sel[i0 + r] of the batch instead of i0 + r (a render's
@@ -237,8 +237,10 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
     const float inv_fs = 1.f / feat_scale;
-    const bool valid = i0 + tid < i_end;
-    const uint32_t i = kSel ? (valid ? sel[i0 + tid] : 0u) : i0 + tid;
+    // which sample a row holds is free: the rows of a warp follow the encoding's pairs
+    const uint32_t ti = i0 + (tid & ~31) + pair_sample(tid & 31);
+    const bool valid = ti < i_end;
+    const uint32_t i = kSel ? (valid ? sel[ti] : 0u) : ti;
     float v[32];
     float3 d = make_float3(0.f, 0.f, 0.f);
     float3 x = make_float3(0.f, 0.f, 0.f);
@@ -246,14 +248,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     // one group of kGatherGroup = 4 levels = 8 features = one 16-byte chunk of the row
 #pragma unroll 1
     for (int g = 0; g < kEnc / 8; ++g) {
-        if (valid) {
-            encode_group(c, tables, x, kGatherGroup * g, v);
+        encode_group(c, tables, x, kGatherGroup * g, v);  // whole warps (an invalid row: position 0)
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] *= feat_scale;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = 0.f;
-        }
+        for (int k = 0; k < 8; ++k) v[k] = valid ? v[k] * feat_scale : 0.f;
         uint4 q;
         q.x = pack2<BF16>(v[0], v[1]);
         q.y = pack2<BF16>(v[2], v[3]);
