@@ -541,6 +541,11 @@ int map_step(map_handle h, uint32_t n_rays, uint64_t seed, uint32_t flags, float
             h->pose_g_cap = cap;
         }
         h->bufs.pose_s = h->pose_s;
+        // the second part of dL/dp: in the half of the encoding buffer that 16-bit rows
+        // leave free, or over the FP32 rows, which the backward has read by then
+        const bool fp32 = h->cfg.precision == MAP_PREC_FP32;
+        h->bufs.pose_odd = reinterpret_cast<float4*>(h->bufs.feat) + (fp32 ? 0 : 4 * h->bufs.cap_samples);
+        h->bufs.pose_odd_stride = fp32 ? 8u : 1u;
         NM_CUDA(h, cudaMemsetAsync(h->pose_g, 0, h->kfs.size() * 8 * sizeof(float), s));
     }
     const StepBufs& b = h->bufs;

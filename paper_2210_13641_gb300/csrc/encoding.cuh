@@ -17,7 +17,7 @@ __device__ __forceinline__ float corner_weight(int k, float wx, float wy, float 
 // and 16 + i (encode_level's loads then cover 16 consecutive samples each).
 __device__ __forceinline__ uint32_t pair_sample(uint32_t lane) { return (lane >> 1) + 16u * (lane & 1u); }
 
-// Features of level l of grid position x into f[0], f[1]; called by all 32 lanes, whose
+// Table values around grid position x at level l; called by all 32 lanes, whose
 // positions follow pair_sample.  tables: [L][T] float2.  The gathers are bound by the
 // 128-byte lines their instructions touch in the L1 (39.5 wavefronts per sample at 73 % of
 // the data pipe when every lane read its own corners, odd x pairs in two instructions).
@@ -27,17 +27,17 @@ __device__ __forceinline__ uint32_t pair_sample(uint32_t lane) { return (lane >>
 // its upper corner by a shuffle.  That is 27.7 lines per sample on the room workload's
 // rays instead of 43.7 (counted on the host); forward of 19.5 M samples 3.36 ms,
 // 3.66 before.  The corners are summed in the order k = 0 .. 7.
-__device__ __forceinline__ void encode_level(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
-                                             float* f) {
+// The 4 (y, z) pairs of this lane's corners (lower and upper in x) and the offsets w.
+__device__ __forceinline__ void level_corners(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
+                                              float2* lo, float2* up, float* w) {
     const uint32_t N = c.res[l], Tmask = c.T - 1;
     const bool dense = (c.dense_mask >> l) & 1u;
     const bool odd = threadIdx.x & 1u;
     const uint32_t m1 = dense ? N + 1u : 2654435761u, m2 = dense ? (N + 1u) * (N + 1u) : 805459861u;
     uint32_t cx, cy, cz;
-    float wx, wy, wz;
-    level_cell(x.x, N, cx, wx);
-    level_cell(x.y, N, cy, wy);
-    level_cell(x.z, N, cz, wz);
+    level_cell(x.x, N, cx, w[0]);
+    level_cell(x.y, N, cy, w[1]);
+    level_cell(x.z, N, cz, w[2]);
     const uint32_t ya = cy * m1, za = cz * m2;
     const uint32_t xn = __shfl_xor_sync(0xffffffffu, cx, 1), yn = __shfl_xor_sync(0xffffffffu, ya, 1),
                    zn = __shfl_xor_sync(0xffffffffu, za, 1);
@@ -55,17 +55,29 @@ __device__ __forceinline__ void encode_level(const DevCfg& c, const float2* __re
             v[i][j] = __ldg(tab + s);
         }
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 snd = odd ? v[0][j] : v[1][j];
+        lo[j] = odd ? v[1][j] : v[0][j];
+        up[j] = make_float2(__shfl_xor_sync(0xffffffffu, snd.x, 1), __shfl_xor_sync(0xffffffffu, snd.y, 1));
+    }
+}
+
+// Features of level l of grid position x into f[0], f[1] (whole warps, pair_sample order).
+__device__ __forceinline__ void encode_level(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
+                                             float* f) {
+    float2 lo[4], up[4];
+    float w[3];
+    level_corners(c, tables, x, l, lo, up, w);
     float a0 = 0.f, a1 = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float2 lo = odd ? v[1][j] : v[0][j], snd = odd ? v[0][j] : v[1][j];
-        const float ux = __shfl_xor_sync(0xffffffffu, snd.x, 1), uy = __shfl_xor_sync(0xffffffffu, snd.y, 1);
-        const float w0 = corner_weight(2 * j, wx, wy, wz);
-        const float w1 = corner_weight(2 * j + 1, wx, wy, wz);
-        a0 += w0 * lo.x;
-        a1 += w0 * lo.y;
-        a0 += w1 * ux;
-        a1 += w1 * uy;
+        const float w0 = corner_weight(2 * j, w[0], w[1], w[2]);
+        const float w1 = corner_weight(2 * j + 1, w[0], w[1], w[2]);
+        a0 += w0 * lo[j].x;
+        a1 += w0 * lo[j].y;
+        a0 += w1 * up[j].x;
+        a1 += w1 * up[j].y;
     }
     f[0] = a0;
     f[1] = a1;
@@ -248,42 +260,39 @@ __device__ __forceinline__ void scatter_tile(const DevCfg& c, float2* __restrict
     else scatter_walk<2, true>(s, gtab, mask, pos, df, n);
 }
 
-// dL/dx = sum_l (d f_l / dx) . dL/df_l at grid position x, for the pose gradient:
-// inside a cell of level l (resolution N) the trilinear weight of corner k is
-// w_k = prod_a (b_a ? w_a : 1 - w_a) with w_a = x_a N - c_a, so
+// dL/dx = sum_l (d f_l / dx) . dL/df_l at grid position x over the levels l0, l0 + 2, ...,
+// for the pose gradient: inside a cell of level l (resolution N) the trilinear weight of
+// corner k is w_k = prod_a (b_a ? w_a : 1 - w_a) with w_a = x_a N - c_a, so
 // dw_k/dx_a = N (b_a ? 1 : -1) prod_{a' != a} (b_a' ? w_a' : 1 - w_a'); the table
-// values of the 8 corners are read again.  df: dL/df [kEnc].
-__device__ __forceinline__ float3 hash_grad_x(const DevCfg& c, const float2* __restrict__ tables, float3 x,
-                                              const float* df) {
-    const uint32_t Tmask = c.T - 1;
+// values of the 8 corners are read again (whole warps, pair_sample order: the encoding's
+// loads).  df(l): dL/df_l of this lane's sample.  The even and the odd levels are summed by
+// different warps (one thread per sample for all of them made the FP16 backward of 4.87 M
+// samples with pose terms 2.79 ms, against 1.11 without; now 2.38).
+template <class DF>
+__device__ __forceinline__ float3 hash_grad_x(const DevCfg& c, const float2* __restrict__ tables, float3 x, DF df,
+                                              int l0) {
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll 1
-    for (int l = 0; l < kEnc / 2; ++l) {
-        if (l >= (int)c.L) break;
-        const uint32_t N = c.res[l];
-        const bool dense = (c.dense_mask >> l) & 1u;
-        uint32_t cx, cy, cz;
-        float wx, wy, wz;
-        level_cell(x.x, N, cx, wx);
-        level_cell(x.y, N, cy, wy);
-        level_cell(x.z, N, cz, wz);
-        const float2* tab = tables + (size_t)l * c.T;
-        const float g0 = df[2 * l], g1 = df[2 * l + 1];
+    for (int l = l0; l < (int)c.L; l += 2) {
+        float2 lo[4], up[4];
+        float w[3];
+        level_corners(c, tables, x, l, lo, up, w);
+        const float2 g = df(l);
         float ax = 0.f, ay = 0.f, az = 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int bx = k & 1, by = (k >> 1) & 1, bz = (k >> 2) & 1;
-            const uint32_t slot = vertex_slot(cx + bx, cy + by, cz + bz, N, dense, Tmask);
-            const float2 v = __ldg(tab + slot);
-            const float e = v.x * g0 + v.y * g1;                    // corner value . dL/df_l
-            const float fx = bx ? wx : 1.f - wx, fy = by ? wy : 1.f - wy, fz = bz ? wz : 1.f - wz;
-            ax += (bx ? e : -e) * fy * fz;
-            ay += (by ? e : -e) * fx * fz;
-            az += (bz ? e : -e) * fx * fy;
+        for (int j = 0; j < 4; ++j) {
+            const int by = j & 1, bz = j >> 1;
+            const float e0 = lo[j].x * g.x + lo[j].y * g.y, e1 = up[j].x * g.x + up[j].y * g.y;
+            const float fy = by ? w[1] : 1.f - w[1], fz = bz ? w[2] : 1.f - w[2];
+            const float m = (1.f - w[0]) * e0 + w[0] * e1;
+            ax += (e1 - e0) * fy * fz;
+            ay += (by ? m : -m) * fz;
+            az += (bz ? m : -m) * fy;
         }
-        gx += (float)N * ax;
-        gy += (float)N * ay;
-        gz += (float)N * az;
+        const float N = small_float(c.res[l]);
+        gx += N * ax;
+        gy += N * ay;
+        gz += N * az;
     }
     return make_float3(gx, gy, gz);
 }

@@ -53,7 +53,9 @@ struct StepBufs {
     float* loss;            // [0] batch loss, [1] [2] largest seeds (FP32 bits), [3] block counter,
                             // bytes 32..39: retained samples of the current render (all chunks)
     float* partials;        // [kCompositeMaxBlocks][4] per-block sums of the compositing kernel
-    float4* pose_s;         // [cap_samples][2] per-sample pose terms (dL/dp, dL/dd via SH); lazily
+    float4* pose_s;         // [cap_samples][2] per-sample pose terms (dL/dp even levels, dL/dd via SH); lazily
+    float4* pose_odd;       // sample i's dL/dp through the odd levels at [pose_odd_stride * i] (in feat)
+    uint32_t pose_odd_stride;
     uint32_t* err;          // [1]
     uint64_t cap_samples;
 };

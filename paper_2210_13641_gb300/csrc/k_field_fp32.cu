@@ -18,18 +18,22 @@ struct SmemW {
     float W5[3 * kHid];           // [c][i]
 };
 
+// 16-byte loads, several in flight (each launch pays this once per block).
 __device__ void load_weights(SmemW& s, const float* __restrict__ mlp) {
-    for (int i = threadIdx.x; i < kW1; i += blockDim.x) s.W1[i] = mlp[kOffW1 + i];
-    for (int i = threadIdx.x; i < kW2; i += blockDim.x) {
-        const int m = i / kHid, j = i % kHid;
-        s.W2T[j * kGeo + m] = mlp[kOffW2 + i];
+#pragma unroll 4
+    for (int q = threadIdx.x; q < kMlpParams / 4; q += blockDim.x) {
+        const float4 w = __ldg(reinterpret_cast<const float4*>(mlp) + q);
+        const float v[4] = {w.x, w.y, w.z, w.w};
+        const int i = 4 * q;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i < kOffW2) s.W1[i + k] = v[k];
+            else if (i < kOffW3) s.W2T[((i - kOffW2) % kHid + k) * kGeo + (i - kOffW2) / kHid] = v[k];
+            else if (i < kOffW4) s.W3[i - kOffW3 + k] = v[k];
+            else if (i < kOffW5) s.W4T[((i - kOffW4) % kHid + k) * kHid + (i - kOffW4) / kHid] = v[k];
+            else s.W5[i - kOffW5 + k] = v[k];
+        }
     }
-    for (int i = threadIdx.x; i < kW3; i += blockDim.x) s.W3[i] = mlp[kOffW3 + i];
-    for (int i = threadIdx.x; i < kW4; i += blockDim.x) {
-        const int r = i / kHid, j = i % kHid;
-        s.W4T[j * kHid + r] = mlp[kOffW4 + i];
-    }
-    for (int i = threadIdx.x; i < kW5; i += blockDim.x) s.W5[i] = mlp[kOffW5 + i];
 }
 
 __device__ __forceinline__ float3 sample_pos(const DevCfg& c, const float* __restrict__ rays,
@@ -296,8 +300,10 @@ __device__ __forceinline__ void put_masked(float* act, const float (*o)[4]) {
         }
 }
 
-// kPose: also writes, per sample, dL/dp (world position) and the view-direction
-// gradient through the SH encoding into pose_s[2 i], pose_s[2 i + 1].
+// kPose: also writes, per sample, dL/dp (world position) through the even levels into
+// pose_s[2 i] and through the odd ones into pose_odd[8 i] (over the sample's row of feat,
+// which its tile has read), and the view-direction gradient through the SH encoding into
+// pose_s[2 i + 1].
 template <bool kPose>
 __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const float* __restrict__ params,
                                                           float* __restrict__ grads,
@@ -305,15 +311,17 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
                                                           const uint32_t* __restrict__ n_total,
                                                           const uint32_t* __restrict__ ray_id,
                                                           const float* __restrict__ ts,
-                                                          const float* __restrict__ feat,
+                                                          const float* feat,
                                                           const float4* __restrict__ dsig_rgb,
-                                                          float4* __restrict__ pose_s) {
+                                                          float4* __restrict__ pose_s, float4* pose_odd) {
     extern __shared__ __align__(16) float smem_raw[];
     SmemBwd& s = *reinterpret_cast<SmemBwd*>(smem_raw);
     const uint32_t n = *n_total;
     if (blockIdx.x * (uint32_t)kTile >= n) return;
     const float* mlp = params + (size_t)c.L * c.T * 2;
-    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) s.W[i] = mlp[i];
+#pragma unroll 5
+    for (int i = threadIdx.x; i < kMlpParams / 4; i += kBwdThreadsF)
+        reinterpret_cast<float4*>(s.W)[i] = __ldg(reinterpret_cast<const float4*>(mlp) + i);
     const float* W1 = s.W + kOffW1;
     const float* W2 = s.W + kOffW2;
     const float* W3 = s.W + kOffW3;
@@ -477,17 +485,15 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
         }
         __syncthreads();
         scatter_tile(c, gtables, tid, level, s.pos[parity], s.df, n - i0);
-        if (kPose && tid < kTile && i0 + tid < n) {
-            float df[kEnc];
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const float2 v = s.df[tile_df(tid, q)];
-                df[2 * q] = v.x;
-                df[2 * q + 1] = v.y;
-            }
-            const float4 x = s.pos[parity][tile_row(tid)];
-            const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params), make_float3(x.x, x.y, x.z), df);
-            pose_s[2 * (size_t)(i0 + tid)] = make_float4(gx.x * c.inv_size, gx.y * c.inv_size, gx.z * c.inv_size, 0.f);
+        if (kPose) {  // dL/dp: warps 0-3 the even levels, 4-7 the odd ones
+            const int odd = tid >> 7;
+            const uint32_t row = (tid & 96) + pair_sample(lane);
+            const float4 x = s.pos[parity][tile_row(row)];
+            const float3 g = hash_grad_x(c, reinterpret_cast<const float2*>(params), make_float3(x.x, x.y, x.z),
+                                         [&](int l) { return s.df[tile_df(row, l)]; }, odd);
+            if (i0 + row < n)
+                (odd ? pose_odd + 8 * (size_t)(i0 + row) : pose_s + 2 * (size_t)(i0 + row))[0] =
+                    make_float4(g.x * c.inv_size, g.y * c.inv_size, g.z * c.inv_size, 0.f);
         }
         // the next tile's inputs go to rows that nobody reads any more, and to the other
         // position buffer; dL/dfeat is written again many barriers later
@@ -535,11 +541,11 @@ void launch_field_bwd_fp32(const DevCfg& c, const float* params, float* grads, u
     if (pose)
         k_field_bwd_fp32<true><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
                                                                  b.offsets + n_rays, b.ray_id, b.t, b.feat, b.dsig_rgb,
-                                                                 b.pose_s);
+                                                                 b.pose_s, b.pose_odd);
     else
         k_field_bwd_fp32<false><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
                                                                   b.offsets + n_rays, b.ray_id, b.t, b.feat,
-                                                                  b.dsig_rgb, nullptr);
+                                                                  b.dsig_rgb, nullptr, nullptr);
 }
 
 }  // namespace nm

@@ -158,33 +158,48 @@ __device__ __forceinline__ void drain_mma(uint64_t* drain_bar) {
     fence_after_sync();
 }
 
+constexpr int kW1B = 64 * 32 * 2, kW2B = 16 * 64 * 2, kW3B = 64 * 32 * 2, kW4B = 64 * 64 * 2, kW5B = 16 * 64 * 2;
+constexpr int kWB = kW1B + kW2B + kW3B + kW4B + kW5B;  // 20480
+constexpr int kT32 = 128 * 32 * 2, kT64 = 128 * 64 * 2, kT16 = 128 * 16 * 2;
+// byte offsets of the weight tiles in the block's shared memory
+constexpr uint32_t kOW1 = 0, kOW2 = kOW1 + kW1B, kOW3 = kOW2 + kW2B, kOW4 = kOW3 + kW3B, kOW5 = kOW4 + kW4B;
+
 // Weight tiles (MLP type) from the FP32 master weights: W1 64x32, W2 16x64,
-// W3 64x32, W4 64x64, W5 padded to 16x64 (rows 3..15 zero).
-template <bool BF16>
-__device__ void load_weight_tiles(const float* __restrict__ mlp, uint8_t* sW1, uint8_t* sW2, uint8_t* sW3,
-                                  uint8_t* sW4, uint8_t* sW5) {
-    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) {
-        const float w = mlp[i];
-        uint8_t* dst;
-        if (i < kOffW2) {
-            dst = sW1 + tile_offset(i / 32, i % 32, 64);
-        } else if (i < kOffW3) {
-            const int j = i - kOffW2;
-            dst = sW2 + tile_offset(j / 64, j % 64, 16);
-        } else if (i < kOffW4) {
-            const int j = i - kOffW3;
-            dst = sW3 + tile_offset(j / 32, j % 32, 64);
-        } else if (i < kOffW5) {
-            const int j = i - kOffW4;
-            dst = sW4 + tile_offset(j / 64, j % 64, 64);
-        } else {
-            const int j = i - kOffW5;
-            dst = sW5 + tile_offset(j / 64, j % 64, 16);
+// W3 64x32, W4 64x64, W5 padded to 16x64 (rows 3..15 zero).  smem: the block's shared
+// memory, whose start holds the tiles; NT threads (tid 0 .. NT - 1).  Every launch pays
+// this once per block before its first tile, so the loads are 16 bytes and up to 7 in
+// flight per thread (one 4-byte load at a time: 30 us of a small render's or step's
+// forward launch).
+template <bool BF16, int NT>
+__device__ void load_weight_tiles(const float* __restrict__ mlp, uint8_t* smem, int tid) {
+    constexpr int kQuads = kMlpParams / 4, kIters = (kQuads + NT - 1) / NT, kBatch = kIters < 7 ? kIters : 7;
+    static_assert(kMlpParams % 4 == 0 && kOffW2 % 4 == 0 && kOffW3 % 4 == 0 && kOffW4 % 4 == 0 && kOffW5 % 4 == 0,
+                  "four weights of one row at a time");
+#pragma unroll 1
+    for (int b = 0; b < kIters; b += kBatch) {
+        float4 w[kBatch];
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const int q = (b + k) * NT + tid;
+            w[k] = q < kQuads ? __ldg(reinterpret_cast<const float4*>(mlp) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        *reinterpret_cast<uint16_t*>(dst) = pack1<BF16>(w);
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) {
+            const int i = 4 * ((b + k) * NT + tid);
+            if (i >= kMlpParams) continue;
+            uint32_t o;
+            if (i < kOffW2) o = kOW1 + tile_offset(i / 32, i % 32, 64);
+            else if (i < kOffW3) o = kOW2 + tile_offset((i - kOffW2) / 64, (i - kOffW2) % 64, 16);
+            else if (i < kOffW4) o = kOW3 + tile_offset((i - kOffW3) / 32, (i - kOffW3) % 32, 64);
+            else if (i < kOffW5) o = kOW4 + tile_offset((i - kOffW4) / 64, (i - kOffW4) % 64, 64);
+            else o = kOW5 + tile_offset((i - kOffW5) / 64, (i - kOffW5) % 64, 16);
+            *reinterpret_cast<uint2*>(smem + o) =
+                make_uint2(pack1<BF16>(w[k].x) | ((uint32_t)pack1<BF16>(w[k].y) << 16),
+                           pack1<BF16>(w[k].z) | ((uint32_t)pack1<BF16>(w[k].w) << 16));
+        }
     }
-    for (int j = 192 + threadIdx.x; j < 16 * 64; j += blockDim.x)
-        *reinterpret_cast<uint16_t*>(sW5 + tile_offset(j / 64, j % 64, 16)) = 0;
+    for (int j = 192 + 4 * tid; j < 16 * 64; j += 4 * NT)
+        *reinterpret_cast<uint2*>(smem + kOW5 + tile_offset(j / 64, j % 64, 16)) = make_uint2(0u, 0u);
 }
 
 __device__ __forceinline__ float3 sample_pos_tc(const DevCfg& c, const float* __restrict__ rays, uint32_t cap,
@@ -194,11 +209,6 @@ __device__ __forceinline__ float3 sample_pos_tc(const DevCfg& c, const float* __
     return grid_pos(c, o, d, t);
 }
 
-constexpr int kW1B = 64 * 32 * 2, kW2B = 16 * 64 * 2, kW3B = 64 * 32 * 2, kW4B = 64 * 64 * 2, kW5B = 16 * 64 * 2;
-constexpr int kWB = kW1B + kW2B + kW3B + kW4B + kW5B;  // 20480
-constexpr int kT32 = 128 * 32 * 2, kT64 = 128 * 64 * 2, kT16 = 128 * 16 * 2;
-// byte offsets of the weight tiles in the block's shared memory
-constexpr uint32_t kOW1 = 0, kOW2 = kOW1 + kW1B, kOW3 = kOW2 + kW2B, kOW4 = kOW3 + kW3B, kOW5 = kOW4 + kW4B;
 using W1K = KMaj<kOW1, 64>;
 using W2K = KMaj<kOW2, 16>;
 using W3K = KMaj<kOW3, 64>;
@@ -362,10 +372,10 @@ __global__ void __launch_bounds__(128, 4) k_field_fwd_tc(DevCfg c, const float* 
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t bar, drain_bar;
     __shared__ uint32_t tslot;
-    load_weight_tiles<BF16>(params + (size_t)c.L * c.T * 2, smem, smem + kW1B, smem + kW1B + kW2B,
-                            smem + kW1B + kW2B + kW3B, smem + kW1B + kW2B + kW3B + kW4B);
-    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
     const uint32_t n = *n_total;
+    if (blockIdx.x * 128u >= n) return;
+    load_weight_tiles<BF16, 128>(params + (size_t)c.L * c.T * 2, smem, threadIdx.x);
+    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
     const uint32_t n_tiles = (n + 127) / 128;
     const float2* tables = reinterpret_cast<const float2*>(params);
     uint32_t phase = 0;
@@ -403,8 +413,9 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
     __shared__ uint32_t tslot;
     __shared__ DevCfg cfg_s;
     __shared__ uint32_t tile0_s[kGroupMaxItems + 1];
-    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
     const uint32_t total = *n_tiles_total;
+    if (blockIdx.x >= total) return;
+    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
     if (threadIdx.x < n_items) tile0_s[threadIdx.x] = items[threadIdx.x].tile0;
     if (threadIdx.x == 0) tile0_s[n_items] = total;
     __syncthreads();
@@ -422,9 +433,7 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
             uint32_t* dst = reinterpret_cast<uint32_t*>(&cfg_s);
             for (uint32_t w = threadIdx.x; w < sizeof(DevCfg) / 4; w += blockDim.x) dst[w] = src[w];
             if (it.params != cur_params)
-                load_weight_tiles<BF16>(it.params + (size_t)it.c.L * it.c.T * 2, smem, smem + kW1B,
-                                        smem + kW1B + kW2B, smem + kW1B + kW2B + kW3B,
-                                        smem + kW1B + kW2B + kW3B + kW4B);
+                load_weight_tiles<BF16, 128>(it.params + (size_t)it.c.L * it.c.T * 2, smem, threadIdx.x);
             cur_params = it.params;
             cur = j;
             to_tensor();      // the weights to the tensor core, the configuration to every thread
@@ -546,11 +555,24 @@ __device__ __forceinline__ void mask_epilogue(uint32_t trow, uint8_t* tile, int 
     }
 }
 
+// dL/dp (world position) through the levels l0, l0 + 2, ... of a tile's samples, by the 128
+// threads r of a warpgroup, to out[stride * sample].
+__device__ __forceinline__ void pose_terms(const DevCfg& c, const float* __restrict__ params, const float4* pos,
+                                           const float2* df, int r, int l0, uint32_t i0, uint32_t n,
+                                           float4* __restrict__ out, uint32_t stride) {
+    const uint32_t row = (r & ~31) + pair_sample(r & 31);
+    const float4 x = pos[tile_row(row)];
+    const float3 g = hash_grad_x(c, reinterpret_cast<const float2*>(params), make_float3(x.x, x.y, x.z),
+                                 [&](int l) { return df[tile_df(row, l)]; }, l0);
+    if (i0 + row < n)
+        out[stride * (size_t)(i0 + row)] = make_float4(g.x * c.inv_size, g.y * c.inv_size, g.z * c.inv_size, 0.f);
+}
+
 }  // namespace
 
-// kPose: also writes, per sample, dL/dp (world position; IO group) and the
-// view-direction gradient through the SH encoding (MLP group) into pose_s[2 i],
-// pose_s[2 i + 1].
+// kPose: also writes, per sample, dL/dp (world position) through the even levels (IO
+// group) into pose_s[2 i] and through the odd ones (SC group) into pose_odd[i], and the
+// view-direction gradient through the SH encoding (MLP group) into pose_s[2 i + 1].
 template <bool BF16, bool kPose>
 __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const float* __restrict__ params,
                                                          float* __restrict__ grads, const float* __restrict__ rays,
@@ -560,15 +582,11 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
                                                          const float4* __restrict__ sig_rgb,
                                                          const float4* __restrict__ dsig_rgb, float feat_scale,
                                                          const float* __restrict__ seed_max,
-                                                         float4* __restrict__ pose_s, uint32_t* __restrict__ err) {
+                                                         float4* __restrict__ pose_s, float4* __restrict__ pose_odd,
+                                                         uint32_t* __restrict__ err) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t bar, drain_bar;
     __shared__ uint32_t tslot;
-    uint8_t* sW1 = smem;
-    uint8_t* sW2 = sW1 + kW1B;
-    uint8_t* sW3 = sW2 + kW2B;
-    uint8_t* sW4 = sW3 + kW3B;
-    uint8_t* sW5 = sW4 + kW4B;
     uint8_t* tX0 = smem + kWB;   // 128 x 32, written by the IO group
     uint8_t* tH1 = tX0 + kT32;   // 128 x 64  (later G1)
     uint8_t* tX3 = tH1 + kT64;   // 128 x 32  (later G2 in columns 0..15)
@@ -595,8 +613,10 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
     using H4M = MnMaj<kOH4, 128>;
     using G5M = MnMaj<kOG5, 128>;
 
+    const uint32_t n = *n_total;
+    if (blockIdx.x * 128u >= n) return;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), r = tid & 127;
-    load_weight_tiles<BF16>(params + (size_t)c.L * c.T * 2, sW1, sW2, sW3, sW4, sW5);
+    load_weight_tiles<BF16, kBwdThreads>(params + (size_t)c.L * c.T * 2, smem, tid);
     if (warp == 0) tmem_alloc(&tslot, 256);
     if (tid == 0) {
         mbar_init(&bar, 1);
@@ -605,7 +625,6 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
     }
     to_tensor();
     const uint32_t tmem = tslot;
-    const uint32_t n = *n_total;
     const uint32_t n_tiles = (n + 127) / 128;
     const uint32_t n_mine = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     const float gm_d = seed_max[1], gm_c = seed_max[2];
@@ -775,8 +794,10 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
         const uint32_t level = scatter_level(c, 128u + r);
         for (uint32_t k = 0; k < n_mine; ++k) {
             nb_sync(kBarDfReady, kBwdThreads);
-            scatter_tile(c, reinterpret_cast<float2*>(grads), 128u + r, level, sX + (k & 1u) * 128, sDf2,
-                         n - (blockIdx.x + k * gridDim.x) * 128);
+            const uint32_t i0 = (blockIdx.x + k * gridDim.x) * 128;
+            const float4* pos = sX + (k & 1u) * 128;
+            scatter_tile(c, reinterpret_cast<float2*>(grads), 128u + r, level, pos, sDf2, n - i0);
+            if (kPose) pose_terms(c, params, pos, sDf2, r, 1, i0, n, pose_odd, 1);
             if (k + 1 < n_mine) nb_arrive(kBarDfFree, kBwdThreads);
         }
         __syncthreads_or(false);                      // pairs with the MLP group's flush barrier
@@ -830,20 +851,7 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             const uint32_t i0 = (blockIdx.x + k * gridDim.x) * 128;
             const float4* pos = sX + (k & 1u) * 128;
             scatter_tile(c, reinterpret_cast<float2*>(grads), r, level, pos, sDf2, n - i0);
-            if (kPose && i0 + r < n) {
-                float v[32];
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const float2 a = sDf2[tile_df(r, q)];
-                    v[2 * q] = a.x;
-                    v[2 * q + 1] = a.y;
-                }
-                const float4 xq = pos[tile_row(r)];
-                const float3 gx = hash_grad_x(c, reinterpret_cast<const float2*>(params),
-                                              make_float3(xq.x, xq.y, xq.z), v);
-                pose_s[2 * (size_t)(i0 + r)] =
-                    make_float4(gx.x * c.inv_size, gx.y * c.inv_size, gx.z * c.inv_size, 0.f);
-            }
+            if (kPose) pose_terms(c, params, pos, sDf2, r, 0, i0, n, pose_s, 2);
             if (k + 1 < n_mine) nb_arrive(kBarDfFree, kBwdThreads);  // dL/dfeat read: the MLP group may overwrite it
         }
         __syncthreads_or(false);                      // pairs with the MLP group's flush barrier
@@ -876,7 +884,7 @@ static void bwd_tc(const DevCfg& c, const float* params, float* grads, uint32_t 
     const float fs = BF16 ? 1.f : 256.f;
     k_field_bwd_tc<BF16, kPose><<<n_sm * 2, kBwdThreads, kBwdSmem, s>>>(
         c, params, grads, b.rays, b.cap_rays, b.offsets + n_rays, b.ray_id, b.t, reinterpret_cast<const uint4*>(b.feat),
-        b.sig_rgb, b.dsig_rgb, fs, b.loss, kPose ? b.pose_s : nullptr, b.err);
+        b.sig_rgb, b.dsig_rgb, fs, b.loss, kPose ? b.pose_s : nullptr, kPose ? b.pose_odd : nullptr, b.err);
 }
 
 template <bool BF16>

@@ -1,6 +1,7 @@
 // k_pose.cu - the keyframe pose gradient of the mapping loss (joint pose refinement:
 // Sec. 3.2 minimises L_M over the poses T as well as the map).  The field backward
-// kernels leave, per sample, dL/dp (the gradient at the sample's world position) and
+// kernels leave, per sample, dL/dp (the gradient at the sample's world position, in two
+// parts) and
 // the view-direction gradient that reaches the sample through its SH encoding; here
 // one warp per ray sums them along the ray (p = o + t d, t fixed), giving dL/do and
 // dL/dd, and turns them into the gradient of the ray's keyframe pose under the left
@@ -18,7 +19,9 @@ constexpr unsigned kFullMask = 0xffffffffu;
 __global__ void __launch_bounds__(256) k_pose_reduce(uint32_t n_rays, const float* __restrict__ rays, uint32_t cap,
                                                      const uint32_t* __restrict__ offsets,
                                                      const float* __restrict__ ts,
-                                                     const float4* __restrict__ pose_s, float* __restrict__ pose_g) {
+                                                     const float4* __restrict__ pose_s,
+                                                     const float4* __restrict__ pose_odd, uint32_t odd_stride,
+                                                     float* __restrict__ pose_g) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
     for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rays; r += n_warps) {
@@ -26,8 +29,12 @@ __global__ void __launch_bounds__(256) k_pose_reduce(uint32_t n_rays, const floa
         if (a == b) continue;  // warp-uniform
         float go[3] = {0.f, 0.f, 0.f}, gd[3] = {0.f, 0.f, 0.f};
         for (uint32_t s = a + lane; s < b; s += 32) {
-            const float4 p = pose_s[2 * s], q = pose_s[2 * s + 1];
+            float4 p = pose_s[2 * (size_t)s];
+            const float4 q = pose_s[2 * (size_t)s + 1], o = pose_odd[odd_stride * (size_t)s];
             const float t = ts[s];
+            p.x += o.x;
+            p.y += o.y;
+            p.z += o.z;
             go[0] += p.x;
             go[1] += p.y;
             go[2] += p.z;
@@ -62,7 +69,8 @@ void launch_pose_reduce(const DevCfg& c, uint32_t n_rays, const StepBufs& b, flo
     (void)c;
     uint32_t grid = (n_rays + 7) / 8;
     if (grid > 152u * 16u) grid = 152u * 16u;
-    k_pose_reduce<<<grid, 256, 0, s>>>(n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.pose_s, pose_g);
+    k_pose_reduce<<<grid, 256, 0, s>>>(n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.pose_s, b.pose_odd, b.pose_odd_stride,
+                                         pose_g);
 }
 
 }  // namespace nm
