@@ -497,7 +497,8 @@ static int run_forward(map_scene* h, uint32_t n_rays, bool train, cudaStream_t s
     const StepBufs& b = h->bufs;
     int rc = phase(h, MAP_PH_MARCH, 5, s, [&] { launch_march(h->dc, h->occ_bits, n_rays, b, s); });
     if (rc) return rc;
-    return phase(h, MAP_PH_FIELD_FWD, 1, s, [&] {
+    const bool split = train && h->cfg.precision != MAP_PREC_FP32 && levels_split(h->dc, n_rays);
+    return phase(h, MAP_PH_FIELD_FWD, split ? 2 : 1, s, [&] {
         if (h->cfg.precision == MAP_PREC_FP32)
             launch_field_fwd_fp32(h->dc, h->params, n_rays, b, train, h->n_sm, s);
         else
@@ -557,7 +558,7 @@ int map_step(map_handle h, uint32_t n_rays, uint64_t seed, uint32_t flags, float
     if (!rc) rc = run_forward(h, n_rays, true, s);
     if (!rc) rc = phase(h, MAP_PH_COMPOSITE, 1, s, [&] { launch_composite(h->dc, n_rays, true, b, s); });
     if (!rc)
-        rc = phase(h, MAP_PH_FIELD_BWD, 1, s, [&] {
+        rc = phase(h, MAP_PH_FIELD_BWD, !pose && h->cfg.precision != MAP_PREC_FP32 && levels_split(h->dc, n_rays) ? 2 : 1, s, [&] {
             if (h->cfg.precision == MAP_PREC_FP32)
                 launch_field_bwd_fp32(h->dc, h->params, h->grads, n_rays, b, h->n_sm, s, pose);
             else

@@ -50,6 +50,9 @@ struct DevCfg {
     uint32_t wait_polls;          // poll limit of each MMA-completion wait (tensor-core kernels)
 };
 
+// First of the levels that a map too large for the L2 takes level by level (at most 8).
+__host__ __device__ __forceinline__ uint32_t split_level(uint32_t L) { return L > 8u ? L - 8u : 0u; }
+
 // Default poll limit of a bounded MMA-completion wait: far beyond any MMA chain's
 // latency, far below a watchdog's reach.
 constexpr uint32_t kWaitPollsDefault = 1u << 24;

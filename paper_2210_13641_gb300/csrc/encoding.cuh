@@ -122,13 +122,15 @@ __device__ __forceinline__ void hash_encode(const DevCfg& c, const float2* __res
 // (counted on the host), against 61.4 in 52.2 for sums over runs of equal cells within
 // a warp, and needs no shuffle at all: the backward of 19.5 M samples takes 4.28 ms
 // instead of 6.74.  It runs at 0.6 of the issue rate, with the integer pipe at 0.57.
+// Walks of G = 16 samples: 8 groups and 2 parities per level, two levels per warp.  With at
+// most 8 levels to scatter (G = 8): 16 groups of 8 samples, one level per warp.
 struct ScatterRole {
-    uint32_t N, m1, m2, g, p;   // resolution, y and z strides (or hash primes), sample group, x parity
-    uint32_t level;
+    uint32_t N, m1, m2, p;      // resolution, y and z strides (or hash primes), x parity
+    uint32_t r0, rd, swz, dx;   // first sample row; first dL/dfeat place; permutation of the walk's rows (and of dL/dfeat's)
     bool dense;
 };
 
-// The level of scatter thread st: each half warp has one.  The dense levels pair up
+// The level of scatter thread st at G = 16: each half warp has one.  The dense levels pair up
 // among themselves (one index arithmetic per warp); the others pair coarse with fine,
 // since a fine level flushes at almost every sample and the slowest warp sets the pace
 // (pairs of neighbours, 14 and 15 in one warp: 4.38 against 3.8 ms for the backward).
@@ -146,25 +148,22 @@ __device__ __forceinline__ uint32_t scatter_level(const DevCfg& c, uint32_t st) 
     return level;
 }
 
-__device__ __forceinline__ ScatterRole scatter_role(const DevCfg& c, uint32_t st, uint32_t level) {
-    ScatterRole s;
-    s.level = level;
-    s.g = (st >> 1) & 7u;
-    s.p = st & 1u;
+__device__ __forceinline__ void set_level(const DevCfg& c, uint32_t level, ScatterRole& s) {
     s.N = c.res[level];
     s.dense = (c.dense_mask >> level) & 1u;
     s.m1 = s.dense ? s.N + 1u : 2654435761u;
     s.m2 = s.dense ? (s.N + 1u) * (s.N + 1u) : 805459861u;
-    return s;
 }
 
 // Physical row of sample row r in the tile buffers the scatter walks (positions, and
-// dL/dfeat per level): lanes of the 8 groups read rows 16 g + i with the same i, which
-// the permutation spreads over all banks (and the odd levels, which mostly share a
-// warp with even ones, over the other half).
-__device__ __forceinline__ uint32_t tile_row(uint32_t r) { return r ^ ((r >> 4) & 7u); }
+// dL/dfeat per level): lanes of the groups read rows G g + i with the same i, which
+// the permutation spreads over all banks (dL/dfeat: the odd levels of G = 16, which mostly
+// share a warp with even ones, or the upper groups of G = 8, over the other half).
+template <int G>
+__device__ __forceinline__ uint32_t tile_row(uint32_t r) { return r ^ ((r / G) & 7u); }
+template <int G>
 __device__ __forceinline__ uint32_t tile_df(uint32_t r, uint32_t level) {
-    return level * 128u + (tile_row(r) ^ ((level & 1u) << 3));
+    return level * 128u + (tile_row<G>(r) ^ ((G == 16 ? level & 1u : (r >> 6) & 1u) << 3));
 }
 
 // Where a differs from b: acc leaves to *p by one 8-byte FP32 reduction, and is cleared.
@@ -192,7 +191,9 @@ template <int kMode, bool kUnit>
 __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __restrict__ gtab, uint32_t mask,
                                              const float4* pos, const float2* df, uint32_t n) {
     const float Nf = small_float(s.N), top = Nf - 0.5f;
-    const uint32_t r0 = 16u * s.g, dswz = s.g ^ ((s.level & 1u) << 3), np = 1u - s.p;
+    const uint32_t np = 1u - s.p;
+    pos += s.r0;
+    df += s.rd;
     const float sx = s.p ? -1.f : 1.f, tx = s.p ? 1.f : 0.f;
     uint32_t held[4];                                     // slots by parity, [2 z + y]
     float2 acc[4];
@@ -203,8 +204,8 @@ __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __res
     }
 #pragma unroll 1
     for (uint32_t i = 0; i < n; ++i) {
-        const float4 q = pos[r0 + (i ^ s.g)];
-        const float2 gl = df[(r0 + i) ^ dswz];
+        const float4 q = pos[i ^ s.swz];
+        const float2 gl = df[i ^ s.swz ^ s.dx];
         const float qx = fmul(q.x, Nf), qy = fmul(q.y, Nf), qz = fmul(q.z, Nf);
         // positions are >= 0 (the box test)
         const uint32_t cx = __float_as_uint(__fadd_rd(fminf(qx, top), 8388608.f));
@@ -243,18 +244,33 @@ __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __res
     for (int k = 0; k < 4; ++k) atomicAdd(gtab + held[k], acc[k]);
 }
 
-// level: scatter_level(c, st); pos: [128] (x, y, z, -) by tile_row; df: dL/dfeat by tile_df; n_valid: samples in the tile.
+__device__ __forceinline__ bool unit_box(const DevCfg& c) {
+    return c.box[0] <= 1.f && c.box[1] <= 1.f && c.box[2] <= 1.f;
+}
+
+// pos: [128] (x, y, z, -) by tile_row; df: dL/dfeat by tile_df; n_valid: samples in the
+// tile; n_levels: the levels 0 .. n_levels - 1 are scattered (G = 8: at most 8).  level:
+// scatter_level(c, st) (G = 16 only).
+template <int G>
 __device__ __forceinline__ void scatter_tile(const DevCfg& c, float2* __restrict__ gtables, uint32_t st,
-                                             uint32_t level, const float4* pos, const float2* df, uint32_t n_valid) {
-    const ScatterRole s = scatter_role(c, st, level);
-    const uint32_t r0 = 16u * s.g;
-    const uint32_t n = level < c.L && r0 < n_valid ? min(16u, n_valid - r0) : 0u;
+                                             uint32_t level, uint32_t n_levels, const float4* pos, const float2* df,
+                                             uint32_t n_valid) {
+    const uint32_t lane = st & 31u;
+    const uint32_t g = G == 16 ? (lane >> 1) & 7u : lane >> 1;
+    if (G == 8) level = st >> 5;
+    ScatterRole s;
+    set_level(c, level, s);
+    s.p = lane & 1u;
+    s.r0 = G * g;
+    s.swz = g & 7u;
+    s.dx = G == 16 ? (level & 1u) << 3 : 0u;
+    s.rd = level * 128u + (G == 16 ? s.r0 : s.r0 ^ ((g >> 3) << 3));
+    const uint32_t n = level < n_levels && s.r0 < n_valid ? min((uint32_t)G, n_valid - s.r0) : 0u;
     const uint32_t hashed = __ballot_sync(0xffffffffu, n && !s.dense), dense = __ballot_sync(0xffffffffu, n && s.dense);
     if (n == 0u) return;
-    float2* gtab = gtables + (size_t)s.level * c.T;
-    df += s.level * 128;
+    float2* gtab = gtables + (size_t)level * c.T;
     const uint32_t mask = c.T - 1;
-    if (!(c.box[0] <= 1.f && c.box[1] <= 1.f && c.box[2] <= 1.f)) scatter_walk<2, false>(s, gtab, mask, pos, df, n);
+    if (!unit_box(c)) scatter_walk<2, false>(s, gtab, mask, pos, df, n);
     else if (dense == 0u) scatter_walk<0, true>(s, gtab, mask, pos, df, n);
     else if (hashed == 0u) scatter_walk<1, true>(s, gtab, mask, pos, df, n);
     else scatter_walk<2, true>(s, gtab, mask, pos, df, n);

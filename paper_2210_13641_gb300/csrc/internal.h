@@ -198,6 +198,9 @@ void launch_field_fwd_tc_sel(const DevCfg& c, const float* params, const uint32_
                              const StepBufs& b, bool bf16, int n_sm, cudaStream_t s);
 void launch_field_fwd_tc(const DevCfg& c, const float* params, uint32_t n_rays, const StepBufs& b,
                          bool store_feat, bool bf16, int n_sm, cudaStream_t s);
+// Whether a step without pose terms takes the finest levels level by level, in a launch of
+// their own (large tables).
+bool levels_split(const DevCfg& c, uint32_t n_rays);
 void launch_field_bwd_tc(const DevCfg& c, const float* params, float* grads, uint32_t n_rays,
                          const StepBufs& b, bool bf16, int n_sm, cudaStream_t s, bool pose = false);
 

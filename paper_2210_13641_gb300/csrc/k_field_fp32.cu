@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
                     x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
                     sh16(d.x, d.y, d.z, sh);
                 }
-                s.pos[parity][tile_row(r)] = make_float4(x.x, x.y, x.z, 0.f);
+                s.pos[parity][tile_row<16>(r)] = make_float4(x.x, x.y, x.z, 0.f);
                 #pragma unroll
                 for (int k = 0; k < 16; k += 4)
                     *reinterpret_cast<float4*>(row + kRx3 + kGeo + k) = make_float4(sh[k], sh[k + 1], sh[k + 2], sh[k + 3]);
@@ -480,17 +480,17 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
         dot_cols<kHid, kEnc, 4>(W1 + 4 * warp, row0 + kRh1, o);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            s.df[tile_df(lane + 32 * q, 2 * warp)] = make_float2(o[0][q], o[1][q]);
-            s.df[tile_df(lane + 32 * q, 2 * warp + 1)] = make_float2(o[2][q], o[3][q]);
+            s.df[tile_df<16>(lane + 32 * q, 2 * warp)] = make_float2(o[0][q], o[1][q]);
+            s.df[tile_df<16>(lane + 32 * q, 2 * warp + 1)] = make_float2(o[2][q], o[3][q]);
         }
         __syncthreads();
-        scatter_tile(c, gtables, tid, level, s.pos[parity], s.df, n - i0);
+        scatter_tile<16>(c, gtables, tid, level, c.L, s.pos[parity], s.df, n - i0);
         if (kPose) {  // dL/dp: warps 0-3 the even levels, 4-7 the odd ones
             const int odd = tid >> 7;
             const uint32_t row = (tid & 96) + pair_sample(lane);
-            const float4 x = s.pos[parity][tile_row(row)];
+            const float4 x = s.pos[parity][tile_row<16>(row)];
             const float3 g = hash_grad_x(c, reinterpret_cast<const float2*>(params), make_float3(x.x, x.y, x.z),
-                                         [&](int l) { return s.df[tile_df(row, l)]; }, odd);
+                                         [&](int l) { return s.df[tile_df<16>(row, l)]; }, odd);
             if (i0 + row < n)
                 (odd ? pose_odd + 8 * (size_t)(i0 + row) : pose_s + 2 * (size_t)(i0 + row))[0] =
                     make_float4(g.x * c.inv_size, g.y * c.inv_size, g.z * c.inv_size, 0.f);

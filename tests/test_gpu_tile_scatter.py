@@ -25,6 +25,11 @@ CASES = [
 ]
 
 
+# tables larger than the L2 and enough rays: the finest levels level by level
+# (9 levels: one of them as usual; 12: four)
+CASES += [(9, 21, 1.9, 4099, 128, 1.0), (12, 21, 1.5, 5000, 128, 1.0)]
+
+
 @pytest.mark.parametrize("prec", ["fp16", "bf16", "fp32"])
 @pytest.mark.parametrize("levels,log2t,growth,rays,smax,box", CASES)
 def test_table_gradient_matches_oracle(prec, levels, log2t, growth, rays, smax, box):
