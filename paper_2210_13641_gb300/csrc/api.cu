@@ -495,7 +495,8 @@ int map_add_keyframe(map_handle h, uint32_t kf_id, const float c2w[12], const fl
 
 static int run_forward(map_scene* h, uint32_t n_rays, bool train, cudaStream_t s) {
     const StepBufs& b = h->bufs;
-    int rc = phase(h, MAP_PH_MARCH, 5, s, [&] { launch_march(h->dc, h->occ_bits, n_rays, b, s); });
+    int rc = phase(h, MAP_PH_MARCH, 2, s,
+                   [&] { launch_march(h->dc, h->occ_bits, n_rays, b, nullptr, nullptr, nullptr, s); });
     if (rc) return rc;
     const bool split = train && h->cfg.precision != MAP_PREC_FP32 && levels_split(h->dc, n_rays);
     return phase(h, MAP_PH_FIELD_FWD, split ? 2 : 1, s, [&] {
@@ -924,11 +925,12 @@ int map_render(map_handle h, const float c2w[12], const float K[4], uint32_t W, 
             if (!rc) rc = phase(h, MAP_PH_COMPOSITE, 1, s, [&] { launch_composite(dc, cnt, false, b, s); });
         } else {
             uint32_t* off = h->render_off;  // off[cnt]: the pass's total, read by the forward
-            if (!rc) rc = phase(h, MAP_PH_MARCH, 5, s, [&] { launch_march(h->dc, h->occ_bits, cnt, b, s); });
+            if (!rc)
+                rc = phase(h, MAP_PH_MARCH, 2, s,
+                           [&] { launch_march(h->dc, h->occ_bits, cnt, b, off, sel, render_eval_counter(b), s); });
             for (int pass = 1; pass <= 2 && !rc; ++pass) {
-                rc = phase(h, MAP_PH_FIELD_FWD, pass == 1 ? 6 : 5, s, [&] {
-                    launch_render_select(cnt, b.offsets, b.counts, pass == 1, kRenderFirst, off, b.block_sums, sel,
-                                         render_eval_counter(b), s);
+                rc = phase(h, MAP_PH_FIELD_FWD, pass, s, [&] {
+                    if (pass == 2) launch_select(cnt, b, b.counts, off, sel, render_eval_counter(b), s);
                     fwd_sel(off + cnt);
                 });
                 if (!rc)

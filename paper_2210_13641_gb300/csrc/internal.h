@@ -32,8 +32,8 @@ enum RayPlane { kOx = 0, kOy, kOz, kDx, kDy, kDz, kIr, kIg, kIb, kD, kV, kKf, kR
 
 constexpr uint32_t kCompositeMaxBlocks = 4096;
 
-// Exclusive scan of per-ray counts (k_rays.cu): one 1024-thread block scans a tile of
-// kScanTile counts and writes the tile's total; a second pass scans the totals.
+// Tile of rays whose sample counts are totalled together; the allocation-free march's scan
+// (k_rays.cu) takes a tile per 1024-thread block.
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;
 constexpr int kScanTile = kScanThreads * kScanPer;
@@ -43,7 +43,7 @@ struct StepBufs {
     uint32_t cap_rays;
     uint32_t* counts;       // [cap_rays]
     uint32_t* offsets;      // [cap_rays + 1] exclusive scan, offsets[n] = total
-    uint32_t* block_sums;   // scan scratch
+    uint32_t* block_sums;   // sample totals per tile of rays
     uint32_t* ray_id;       // [cap_samples]
     float* t;               // [cap_samples]
     float4* sig_rgb;        // [cap_samples] sigma, r, g, b
@@ -72,14 +72,12 @@ inline unsigned long long* render_eval_counter(const StepBufs& b) {
 // A render evaluates the field for the first kSplitFirst samples of every ray, then
 // only for the rays whose transmittance is still above the threshold (k_composite.cu).
 constexpr uint32_t kRenderFirst = 32;
-// k_rays.cu: the selection of a pass's samples.  first_pass: count[r] = min(first,
-// samples of ray r), samples 0 .. count[r] - 1 of each ray; otherwise count[r] is given
-// (the composite's live counts) and the samples first .. first + count[r] - 1 are taken.
-// sel_off: [n_rays + 1] (sel_off[n_rays] = the pass's total), tile_sums: scan scratch,
-// sel: the selected sample indices; evaluated accumulates the totals.
-void launch_render_select(uint32_t n_rays, const uint32_t* offsets, uint32_t* count, bool first_pass,
-                          uint32_t first, uint32_t* sel_off, uint32_t* tile_sums, uint32_t* sel,
-                          unsigned long long* evaluated, cudaStream_t s);
+// k_rays.cu: the selection of the second pass: live[r] (the composite's live counts)
+// samples of ray r from its sample kRenderFirst on.  sel_off: [n_rays + 1]
+// (sel_off[n_rays] = the pass's total), sel: the selected sample indices; evaluated
+// accumulates the totals.  (The first pass's selection comes with the march.)
+void launch_select(uint32_t n_rays, const StepBufs& b, const uint32_t* live, uint32_t* sel_off, uint32_t* sel,
+                   unsigned long long* evaluated, cudaStream_t s);
 // k_composite.cu: pass 1 (first kRenderFirst samples, live counts out) or pass 2 (the
 // live rays, from their first sample).
 void launch_composite_split(const DevCfg& c, uint32_t n_rays, int pass, uint32_t* live, const StepBufs& b,
@@ -169,15 +167,16 @@ void launch_ray_gen(const KfDesc* kfs, const uint32_t* active, uint32_t n_kf, ui
                     uint32_t n_rays, const StepBufs& b, cudaStream_t s);
 void launch_ray_gen_view(const float* c2w, const float* K, uint32_t W, uint32_t p0, uint32_t cnt,
                          const StepBufs& b, cudaStream_t s);
-void launch_march(const DevCfg& c, const uint32_t* occ_bits, uint32_t n_rays, const StepBufs& b,
-                  cudaStream_t s);
+// March, offsets and compaction; with sel also the selection of a render's first pass (the
+// first kRenderFirst samples of each ray; as launch_select).
+void launch_march(const DevCfg& c, const uint32_t* occ_bits, uint32_t n_rays, const StepBufs& b, uint32_t* sel_off,
+                  uint32_t* sel, unsigned long long* evaluated, cudaStream_t s);
+
+// k_compact alone (launch_march's second half), slot rows of row_stride floats.
+void launch_compact(uint32_t n_rays, uint32_t row_stride, const StepBufs& b, const float* slots, uint32_t* sel_off,
+                    uint32_t* sel, unsigned long long* evaluated, cudaStream_t s);
 
 // tile_sums: at least ceil(n / kScanTile) words.
-// k_compact: each ray's retained steps from its slot row (row_stride floats per ray)
-// to its scanned offset, with the ray index beside each sample.
-void launch_compact(uint32_t n_rays, uint32_t row_stride, const uint32_t* offsets, const float* slots,
-                    uint32_t* ray_id, float* ts, cudaStream_t s);
-
 void launch_scan_counts(const uint32_t* counts, uint32_t n, uint32_t* offsets, uint32_t* tile_sums,
                         cudaStream_t s);
 

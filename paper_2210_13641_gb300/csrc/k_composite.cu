@@ -5,6 +5,7 @@
 // transmittance exponent is a warp prefix sum carried from chunk to chunk, and the
 // backward's suffix sums are warp suffix scans over the chunks in reverse order.
 #include "internal.h"
+#include "rays.cuh"
 
 namespace nm {
 
@@ -64,7 +65,7 @@ __device__ __forceinline__ float warp_suffix(float x, uint32_t lane) {
 // kSplit (render only) composites in two passes around the forward's two passes:
 // 1 takes the first kRenderFirst samples of each ray and writes, per ray, the number of
 // samples still to evaluate into `live` (0 when the ray stopped at the threshold or
-// has no more samples); 2 takes the rays with live > 0 from their first sample to
+// has no more samples) and adds it to the totals of the ray's tile; 2 takes the rays with live > 0 from their first sample to
 // their last.  A ray is composited in 32-sample chunks from its first sample in
 // every pass, so each result equals the single pass's.
 static_assert(kRenderFirst % 32 == 0, "the first pass must end at a chunk boundary of the compositing");
@@ -74,7 +75,8 @@ __global__ void __launch_bounds__(kCompositeWarps * 32) k_composite(
     DevCfg c, uint32_t n_rays, const float* __restrict__ rays, uint32_t cap, const uint32_t* __restrict__ offsets,
     const float* __restrict__ ts, const float4* __restrict__ sig_rgb, float4* __restrict__ scratch,
     float* __restrict__ ray_out, float* __restrict__ loss, float* __restrict__ partials,
-    const GroupItem* __restrict__ items = nullptr, uint32_t* __restrict__ live = nullptr) {
+    const GroupItem* __restrict__ items = nullptr, uint32_t* __restrict__ live = nullptr,
+    uint32_t* __restrict__ live_totals = nullptr) {
     static_assert(!(kBackward && kGroup), "grouped compositing is forward only");
     static_assert(!(kBackward && kSplit), "two-pass compositing is forward only");
     const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
@@ -120,7 +122,11 @@ __global__ void __launch_bounds__(kCompositeWarps * 32) k_composite(
                 break;
             }
         }
-        if (kSplit == 1 && lane == 0) live[r] = stopped ? 0u : b_all - b;
+        if (kSplit == 1 && lane == 0) {
+            const uint32_t left = stopped ? 0u : b_all - b;
+            live[r] = left;
+            if (left) atomicAdd(live_totals + r / kScanTile, left);
+        }
         Ir = warp_sum(Ir);
         Ig = warp_sum(Ig);
         Ib = warp_sum(Ib);
@@ -248,7 +254,7 @@ void launch_composite_group(const GroupItem* items, uint32_t n_rays, const StepB
     else if (pass == 1)
         k_composite<false, true, 1><<<grid, kCompositeWarps * 32, 0, s>>>(
             unused, n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.sig_rgb, nullptr, b.ray_out, nullptr, nullptr, items,
-            live);
+            live, tile_totals(b, true).live);
     else
         k_composite<false, true, 2><<<grid, kCompositeWarps * 32, 0, s>>>(
             unused, n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.sig_rgb, nullptr, b.ray_out, nullptr, nullptr, items,
@@ -261,7 +267,7 @@ void launch_composite_split(const DevCfg& c, uint32_t n_rays, int pass, uint32_t
     if (pass == 1)
         k_composite<false, false, 1><<<grid, kCompositeWarps * 32, 0, s>>>(
             c, n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.sig_rgb, nullptr, b.ray_out, nullptr, nullptr, nullptr,
-            live);
+            live, tile_totals(b, true).live);
     else
         k_composite<false, false, 2><<<grid, kCompositeWarps * 32, 0, s>>>(
             c, n_rays, b.rays, b.cap_rays, b.offsets, b.t, b.sig_rgb, nullptr, b.ray_out, nullptr, nullptr, nullptr,
@@ -272,7 +278,6 @@ void launch_composite(const DevCfg& c, uint32_t n_rays, bool backward, const Ste
                       cudaStream_t s) {
     const uint32_t grid = composite_grid(n_rays);
     if (backward) {
-        cudaMemsetAsync(b.loss, 0, 4 * sizeof(float), s);
         k_composite<true><<<grid, kCompositeWarps * 32, 0, s>>>(c, n_rays, b.rays, b.cap_rays, b.offsets, b.t,
                                                                 b.sig_rgb, b.dsig_rgb, b.ray_out, b.loss,
                                                                 b.partials);

@@ -38,8 +38,9 @@ __device__ __forceinline__ uint32_t piece_of(const GroupItem* __restrict__ items
 }
 
 __global__ void k_group_raygen(const GroupItem* __restrict__ items, uint32_t n_items, uint32_t n_rays,
-                               float* __restrict__ rays, uint32_t cap) {
+                               float* __restrict__ rays, uint32_t cap, TileTotals totals) {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    clear_totals(totals, r, n_rays);
     if (r >= n_rays) return;
     const uint32_t j = piece_of(items, n_items, r);
     const GroupItem& it = items[j];
@@ -49,40 +50,19 @@ __global__ void k_group_raygen(const GroupItem* __restrict__ items, uint32_t n_i
     store_ray(rays, cap, r, o, d, make_float4(0.f, 0.f, 0.f, 0.f), 1.f, j);
 }
 
-// The march of k_march (one warp per ray, 32 consecutive steps per ballot, the
-// conservative box step range first), with each ray's configuration and bitfield
-// taken from its piece; slot rows of row_stride floats.
-__global__ void k_group_march(const GroupItem* __restrict__ items, uint32_t n_rays, const float* __restrict__ rays,
-                              uint32_t cap, uint32_t* __restrict__ counts, float* __restrict__ slots,
-                              uint32_t row_stride) {
-    const uint32_t lane = threadIdx.x & 31u;
+// The march of k_march, with each ray's configuration and bitfield taken from its piece;
+// slot rows of row_stride floats.
+__global__ void __launch_bounds__(256) k_group_march(const GroupItem* __restrict__ items, uint32_t n_rays,
+                                                     const float* __restrict__ rays, uint32_t cap,
+                                                     uint32_t* __restrict__ counts, float* __restrict__ slots,
+                                                     uint32_t row_stride, TileTotals totals) {
     const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (r >= n_rays) return;  // whole warps
-    const GroupItem& it = items[__float_as_uint(rays[kKf * cap + r])];
-    const DevCfg& c = it.c;
-    const uint32_t* bits = it.occ;
-    const float3 o = make_float3(rays[kOx * cap + r], rays[kOy * cap + r], rays[kOz * cap + r]);
-    const float3 d = make_float3(rays[kDx * cap + r], rays[kDy * cap + r], rays[kDz * cap + r]);
-    float* row = slots + (size_t)r * row_stride;
-    const uint32_t max_samples = c.max_samples;
-    uint32_t i_lo, i_hi;
-    box_step_range(c, o, d, i_lo, i_hi);
     uint32_t n = 0;
-    for (uint32_t i0 = i_lo; i0 < i_hi && n < max_samples; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        bool keep = false;
-        float t = 0.f;
-        if (i < i_hi) {
-            t = sample_t(c, i);
-            const float3 x = grid_pos(c, o, d, t);
-            keep = in_box(c, x) && occupied(c, bits, x);
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, keep);
-        const uint32_t pos = n + __popc(m & ((1u << lane) - 1u));
-        if (keep && pos < max_samples) row[pos] = t;
-        n += __popc(m);
+    if (r < n_rays) {  // whole warps
+        const GroupItem& it = items[__float_as_uint(rays[kKf * cap + r])];
+        n = march_ray(it.c, it.occ, rays, cap, r, slots + (size_t)r * row_stride);
     }
-    if (lane == 0) counts[r] = n < max_samples ? n : max_samples;
+    ray_totals(totals, r, n, n_rays, counts);
 }
 
 // After a scan over the rays (the march's, or a render pass's selection): each
@@ -128,6 +108,7 @@ int group_bufs_alloc(GroupBufs& g, uint32_t cap_rays, uint32_t row_stride) {
         {(void**)&g.sel, sizeof(uint32_t) * cs},
         {(void**)&g.sel_off, sizeof(uint32_t) * (cap_rays + 1)},
         {(void**)&b.loss, 64},
+        {(void**)&b.partials, sizeof(float) * 4 * kCompositeMaxBlocks},
     };
     for (auto& r : reqs) {
         if (cudaMalloc(r.p, r.bytes) != cudaSuccess) {
@@ -148,7 +129,7 @@ int group_bufs_alloc(GroupBufs& g, uint32_t cap_rays, uint32_t row_stride) {
 
 void group_bufs_free(GroupBufs& g) {
     void* ps[] = {g.b.rays, g.b.counts, g.b.offsets, g.b.block_sums, g.b.ray_id, g.b.t, g.b.sig_rgb,
-                  g.b.ray_out, g.b.err, g.items, g.n_tiles, g.sel, g.sel_off, g.b.loss};
+                  g.b.ray_out, g.b.err, g.items, g.n_tiles, g.sel, g.sel_off, g.b.loss, g.b.partials};
     for (void* p : ps)
         if (p) cudaFree(p);
     g = GroupBufs{};
@@ -191,28 +172,27 @@ int render_group(const GroupView* views, uint32_t n, bool bf16, GroupBufs& g, in
             }
         }
         k_set_group_items<<<1, kGroupMaxItems, 0, s>>>(its, n_items, g.items);
-        k_group_raygen<<<(rays + 255) / 256, 256, 0, s>>>(g.items, n_items, rays, b.rays, b.cap_rays);
+        k_group_raygen<<<(rays + 255) / 256, 256, 0, s>>>(g.items, n_items, rays, b.rays, b.cap_rays,
+                                                          tile_totals(b, true));
         float* slots = reinterpret_cast<float*>(b.sig_rgb);
         k_group_march<<<(rays + 7) / 8, 256, 0, s>>>(g.items, rays, b.rays, b.cap_rays, b.counts, slots,
-                                                     g.row_stride);
-        launch_scan_counts(b.counts, rays, b.offsets, b.block_sums, s);
-        launch_compact(rays, g.row_stride, b.offsets, slots, b.ray_id, b.t, s);
+                                                     g.row_stride, tile_totals(b, true));
+        launch_compact(rays, g.row_stride, b, slots, g.sel_off, two_pass ? g.sel : nullptr, render_eval_counter(b), s);
         if (!two_pass) {
             k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, b.offsets, g.n_tiles);
             launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s);
             launch_composite_group(g.items, rays, b, s);
-            if (launches) *launches += 11;  // items, rays, march, 3 scan passes, compaction, tiles, field, composite, write
+            if (launches) *launches += 8;  // items, rays, march, compaction, tiles, field, composite, write
         } else {
             // as map_render: the field for the first kRenderFirst samples of every ray,
             // then for the rays still above their threshold (pieces index the selection)
             for (int pass = 1; pass <= 2; ++pass) {
-                launch_render_select(rays, b.offsets, b.counts, pass == 1, kRenderFirst, g.sel_off, b.block_sums,
-                                     g.sel, render_eval_counter(b), s);
+                if (pass == 2) launch_select(rays, b, b.counts, g.sel_off, g.sel, render_eval_counter(b), s);
                 k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, g.sel_off, g.n_tiles);
                 launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s, g.sel);
                 launch_composite_group(g.items, rays, b, s, pass, b.counts);
             }
-            if (launches) *launches += 23;
+            if (launches) *launches += 12;
         }
         launch_write_group(g.items, rays, b, s);
         if (cudaGetLastError() != cudaSuccess) return MAP_ECUDA;

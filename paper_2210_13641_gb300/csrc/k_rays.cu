@@ -49,8 +49,10 @@ void launch_keyframe_texels(const float* rgb, const float* depth, const float* v
 // list (keyframes streamed out to the host are not drawn) the k-th active keyframe is
 // slot active[k]; without one, slot k.
 __global__ void k_ray_gen(const KfDesc* __restrict__ kfs, const uint32_t* __restrict__ active, uint32_t n_kf,
-                          uint64_t seed, uint64_t step, uint32_t n_rays, float* __restrict__ rays, uint32_t cap) {
+                          uint64_t seed, uint64_t step, uint32_t n_rays, float* __restrict__ rays, uint32_t cap,
+                          TileTotals totals) {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    clear_totals(totals, r, n_rays);
     if (r >= n_rays) return;
     const uint64_t r0 = counter_rand(seed, step, r, 0);
     const uint64_t r1 = counter_rand(seed, step, r, 1);
@@ -69,7 +71,7 @@ __global__ void k_ray_gen(const KfDesc* __restrict__ kfs, const uint32_t* __rest
 void launch_ray_gen(const KfDesc* kfs, const uint32_t* active, uint32_t n_kf, uint64_t seed, uint64_t step,
                     uint32_t n_rays, const StepBufs& b, cudaStream_t s) {
     k_ray_gen<<<(n_rays + 255) / 256, 256, 0, s>>>(kfs, active, n_kf, seed, step, n_rays, b.rays,
-                                                   b.cap_rays);
+                                                   b.cap_rays, tile_totals(b, false));
 }
 
 struct ViewCam {
@@ -79,8 +81,9 @@ struct ViewCam {
 
 // Rays of pixels p0 .. p0 + cnt - 1 of a W-wide view (row-major), as rays 0 .. cnt - 1.
 __global__ void k_ray_gen_view(ViewCam cam, uint32_t W, uint32_t p0, uint32_t cnt, float* __restrict__ rays,
-                               uint32_t cap) {
+                               uint32_t cap, TileTotals totals) {
     const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
+    clear_totals(totals, r, cnt);
     if (r >= cnt) return;
     const uint32_t pix = p0 + r;
     float3 o, d;
@@ -93,54 +96,130 @@ void launch_ray_gen_view(const float* c2w, const float* K, uint32_t W, uint32_t 
     ViewCam cam;
     for (int i = 0; i < 12; ++i) cam.c2w[i] = c2w[i];
     for (int i = 0; i < 4; ++i) cam.K[i] = K[i];
-    k_ray_gen_view<<<(cnt + 255) / 256, 256, 0, s>>>(cam, W, p0, cnt, b.rays, b.cap_rays);
+    k_ray_gen_view<<<(cnt + 255) / 256, 256, 0, s>>>(cam, W, p0, cnt, b.rays, b.cap_rays, tile_totals(b, true));
 }
 
 // ---------------------------------------------------------------- march
 // One pass over the steps of each ray, one warp per ray: the 32 lanes test 32
 // consecutive steps at a time and a ballot gives each retained step its place in
 // the ray's slot row (max_samples floats per ray, in step order); the count goes to
-// counts[r].  After the scan, k_compact copies each ray's row to its offset (one
-// warp per ray, coalesced) and writes the ray index beside each sample.
-__global__ void k_march(DevCfg c, const uint32_t* __restrict__ bits, uint32_t n_rays,
-                        const float* __restrict__ rays, uint32_t cap, uint32_t* __restrict__ counts,
-                        float* __restrict__ slots) {
-    const uint32_t lane = threadIdx.x & 31u;
+// counts[r] and into the totals of the ray's tile (ray_totals).  k_compact then turns the
+// counts into offsets and copies the rows.
+__global__ void __launch_bounds__(256) k_march(DevCfg c, const uint32_t* __restrict__ bits, uint32_t n_rays,
+                                               const float* __restrict__ rays, uint32_t cap,
+                                               uint32_t* __restrict__ counts, float* __restrict__ slots,
+                                               TileTotals totals) {
     const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (r >= n_rays) return;  // whole warps
-    const float3 o = make_float3(rays[kOx * cap + r], rays[kOy * cap + r], rays[kOz * cap + r]);
-    const float3 d = make_float3(rays[kDx * cap + r], rays[kDy * cap + r], rays[kDz * cap + r]);
-    float* row = slots + (size_t)r * c.max_samples;
-    uint32_t i_lo, i_hi;
-    box_step_range(c, o, d, i_lo, i_hi);
     uint32_t n = 0;
-    for (uint32_t i0 = i_lo; i0 < i_hi && n < c.max_samples; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        bool keep = false;
-        float t = 0.f;
-        if (i < i_hi) {
-            t = sample_t(c, i);
-            const float3 x = grid_pos(c, o, d, t);
-            keep = in_box(c, x) && occupied(c, bits, x);
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, keep);
-        const uint32_t pos = n + __popc(m & ((1u << lane) - 1u));
-        if (keep && pos < c.max_samples) row[pos] = t;
-        n += __popc(m);
-    }
-    if (lane == 0) counts[r] = n < c.max_samples ? n : c.max_samples;
+    if (r < n_rays) n = march_ray(c, bits, rays, cap, r, slots + (size_t)r * c.max_samples);  // whole warps
+    ray_totals(totals, r, n, n_rays, counts);
 }
 
-__global__ void k_compact(uint32_t n_rays, uint32_t max_samples, const uint32_t* __restrict__ offsets,
-                          const float* __restrict__ slots, uint32_t* __restrict__ ray_id, float* __restrict__ ts) {
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t lane = threadIdx.x & 31u;
-    if (r >= n_rays) return;
-    const uint32_t a = offsets[r], n = offsets[r + 1] - a;
-    const float* row = slots + (size_t)r * max_samples;
-    for (uint32_t k = lane; k < n; k += 32) {
-        ts[a + k] = row[k];
-        ray_id[a + k] = r;
+// Offsets and compaction: a block takes 64 rays.  What comes before them is the sum of the
+// totals of the tiles before theirs and of the counts before them in their tile, so one
+// launch does what a scan in three and a copy did.  Writes the rays' offsets (and
+// offsets[n_rays]) and copies each ray's row to its offset, with the ray index beside
+// each sample.  kFirst (render): also the first pass's selection, the first
+// min(kRenderFirst, count) samples of each ray (sel_off: its total at [n_rays]).
+constexpr uint32_t kCompactRays = 64;
+
+template <class F>
+__device__ __forceinline__ uint32_t sum_before(const uint32_t* __restrict__ totals, const uint32_t* __restrict__ counts,
+                                               uint32_t r0, F f, uint32_t* warp_sums) {
+    const uint32_t tile = r0 / kScanTile, lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    uint32_t v = 0;
+    for (uint32_t i = threadIdx.x; i < tile; i += 256u) v += totals[i];
+    for (uint32_t i = tile * kScanTile + threadIdx.x; i < r0; i += 256u) v += f(counts[i]);
+    v = __reduce_add_sync(0xffffffffu, v);
+    __syncthreads();
+    if (lane == 0) warp_sums[w] = v;
+    __syncthreads();
+    uint32_t total = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) total += warp_sums[k];
+    return total;
+}
+
+// off[0 .. 64] = base + exclusive scan of v (thread t < 64: ray t's count); 256 threads.
+__device__ __forceinline__ void scan64(uint32_t v, uint32_t base, uint32_t* off) {
+    if (threadIdx.x < kCompactRays) off[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const uint32_t lane = threadIdx.x, a = off[2 * lane], b = off[2 * lane + 1];
+        uint32_t x = a + b;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= (uint32_t)o) x += y;
+        }
+        __syncwarp();
+        off[2 * lane] = base + x - a - b;
+        off[2 * lane + 1] = base + x - b;
+        if (lane == 31) off[64] = base + x;
+    }
+    __syncthreads();
+}
+
+template <bool kFirst>
+__global__ void __launch_bounds__(256) k_compact(uint32_t n_rays, uint32_t row_stride, const uint32_t* __restrict__ counts,
+                                                 TileTotals totals, uint32_t* __restrict__ offsets,
+                                                 const float* __restrict__ slots, uint32_t* __restrict__ ray_id,
+                                                 float* __restrict__ ts, uint32_t* __restrict__ sel_off,
+                                                 uint32_t* __restrict__ sel, unsigned long long* __restrict__ evaluated) {
+    __shared__ uint32_t warp_sums[8], off[kCompactRays + 1], first[kCompactRays + 1];
+    const uint32_t r0 = blockIdx.x * kCompactRays, lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    const uint32_t r = r0 + threadIdx.x;
+    const uint32_t n = threadIdx.x < kCompactRays && r < n_rays ? counts[r] : 0u;
+    scan64(n, sum_before(totals.all, counts, r0, [](uint32_t v) { return v; }, warp_sums), off);
+    if (kFirst)
+        scan64(min(n, kRenderFirst),
+               sum_before(totals.first, counts, r0, [](uint32_t v) { return min(v, kRenderFirst); }, warp_sums), first);
+    if (threadIdx.x < kCompactRays && r < n_rays) {
+        offsets[r] = off[threadIdx.x];
+        if (kFirst) sel_off[r] = first[threadIdx.x];
+        if (r == n_rays - 1) {
+            offsets[n_rays] = off[threadIdx.x + 1];
+            if (kFirst) {
+                sel_off[n_rays] = first[threadIdx.x + 1];
+                atomicAdd(evaluated, (unsigned long long)first[threadIdx.x + 1]);
+            }
+        }
+    }
+    for (uint32_t q = w; q < kCompactRays && r0 + q < n_rays; q += 8u) {
+        const uint32_t a = off[q], m = off[q + 1] - a;
+        const float* row = slots + (size_t)(r0 + q) * row_stride;
+        for (uint32_t k = lane; k < m; k += 32) {
+            ts[a + k] = row[k];
+            ray_id[a + k] = r0 + q;
+        }
+        if (kFirst && lane < first[q + 1] - first[q]) sel[first[q] + lane] = a + lane;
+    }
+}
+static_assert(kRenderFirst <= 32, "k_compact emits a ray's first samples with one warp store");
+
+// Selection of a render's second pass: ray r contributes its live[r] samples from its
+// sample kRenderFirst on, at sel[sel_off[r] ...].
+__global__ void __launch_bounds__(256) k_select(uint32_t n_rays, const uint32_t* __restrict__ offsets,
+                                                const uint32_t* __restrict__ live, TileTotals totals,
+                                                uint32_t* __restrict__ sel_off, uint32_t* __restrict__ sel,
+                                                unsigned long long* __restrict__ evaluated) {
+    __shared__ uint32_t warp_sums[8], off[kCompactRays + 1];
+    const uint32_t r0 = blockIdx.x * kCompactRays, lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    const uint32_t r = r0 + threadIdx.x;
+    const uint32_t n = threadIdx.x < kCompactRays && r < n_rays ? live[r] : 0u;
+    scan64(n, sum_before(totals.live, live, r0, [](uint32_t v) { return v; }, warp_sums), off);
+    if (threadIdx.x < kCompactRays && r < n_rays) {
+        sel_off[r] = off[threadIdx.x];
+        if (r == n_rays - 1) {
+            sel_off[n_rays] = off[threadIdx.x + 1];
+            atomicAdd(evaluated, (unsigned long long)off[threadIdx.x + 1]);
+        }
+    }
+    for (uint32_t q = w; q < kCompactRays && r0 + q < n_rays; q += 8u) {
+        const uint32_t a = off[q], m = off[q + 1] - a;
+        if (m == 0) continue;
+        const uint32_t src = offsets[r0 + q] + kRenderFirst;
+        for (uint32_t k = lane; k < m; k += 32) sel[a + k] = src + k;
     }
 }
 
@@ -225,52 +304,30 @@ __global__ void k_scan_add(uint32_t* __restrict__ out, uint32_t n,
     if (i < n) out[i] += tile_sums[i / kScanTile];
 }
 
-// Selection of a render pass's samples: ray r contributes count[r] samples, its samples
-// k0 .. k0 + count[r] - 1 (counted from its first), at sel[sel_off[r] ...].
-__global__ void k_sel_emit(uint32_t n_rays, const uint32_t* __restrict__ offsets,
-                           const uint32_t* __restrict__ sel_off, const uint32_t* __restrict__ count, uint32_t k0,
-                           uint32_t* __restrict__ sel, unsigned long long* __restrict__ evaluated) {
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t lane = threadIdx.x & 31u;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(evaluated, (unsigned long long)sel_off[n_rays]);
-    if (r >= n_rays) return;
-    const uint32_t n = count[r], dst = sel_off[r], src = offsets[r] + k0;
-    for (uint32_t k = lane; k < n; k += 32) sel[dst + k] = src + k;
+void launch_select(uint32_t n_rays, const StepBufs& b, const uint32_t* live, uint32_t* sel_off, uint32_t* sel,
+                   unsigned long long* evaluated, cudaStream_t s) {
+    k_select<<<(n_rays + kCompactRays - 1) / kCompactRays, 256, 0, s>>>(n_rays, b.offsets, live, tile_totals(b, true),
+                                                                        sel_off, sel, evaluated);
 }
 
-// count[r] = min(first, samples of ray r): the first pass's share of each ray.
-__global__ void k_sel_first(uint32_t n_rays, const uint32_t* __restrict__ offsets, uint32_t first,
-                            uint32_t* __restrict__ count) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rays) return;
-    const uint32_t n = offsets[r + 1] - offsets[r];
-    count[r] = n < first ? n : first;
+void launch_compact(uint32_t n_rays, uint32_t row_stride, const StepBufs& b, const float* slots, uint32_t* sel_off,
+                    uint32_t* sel, unsigned long long* evaluated, cudaStream_t s) {
+    const uint32_t grid = (n_rays + kCompactRays - 1) / kCompactRays;
+    if (sel)
+        k_compact<true><<<grid, 256, 0, s>>>(n_rays, row_stride, b.counts, tile_totals(b, true), b.offsets, slots, b.ray_id,
+                                             b.t, sel_off, sel, evaluated);
+    else
+        k_compact<false><<<grid, 256, 0, s>>>(n_rays, row_stride, b.counts, tile_totals(b, false), b.offsets, slots,
+                                              b.ray_id, b.t, nullptr, nullptr, nullptr);
 }
 
-void launch_render_select(uint32_t n_rays, const uint32_t* offsets, uint32_t* count, bool first_pass,
-                          uint32_t first, uint32_t* sel_off, uint32_t* tile_sums, uint32_t* sel,
-                          unsigned long long* evaluated, cudaStream_t s) {
-    if (first_pass) k_sel_first<<<(n_rays + 255) / 256, 256, 0, s>>>(n_rays, offsets, first, count);
-    launch_scan_counts(count, n_rays, sel_off, tile_sums, s);
-    k_sel_emit<<<(n_rays + 7) / 8, 256, 0, s>>>(n_rays, offsets, sel_off, count, first_pass ? 0u : first, sel,
-                                                 evaluated);
-}
-
-void launch_compact(uint32_t n_rays, uint32_t row_stride, const uint32_t* offsets, const float* slots,
-                    uint32_t* ray_id, float* ts, cudaStream_t s) {
-    k_compact<<<(n_rays + 7) / 8, 256, 0, s>>>(n_rays, row_stride, offsets, slots, ray_id, ts);
-}
-
-void launch_march(const DevCfg& c, const uint32_t* occ_bits, uint32_t n_rays, const StepBufs& b,
-                  cudaStream_t s) {
+void launch_march(const DevCfg& c, const uint32_t* occ_bits, uint32_t n_rays, const StepBufs& b, uint32_t* sel_off,
+                  uint32_t* sel, unsigned long long* evaluated, cudaStream_t s) {
     // slot rows live in the (not yet used) per-sample colour buffer: cap_samples floats
     float* slots = reinterpret_cast<float*>(b.sig_rgb);
-    k_march<<<(n_rays + 7) / 8, 256, 0, s>>>(c, occ_bits, n_rays, b.rays, b.cap_rays, b.counts, slots);
-    const uint32_t n_tiles = (n_rays + kScanTile - 1) / kScanTile;  // <= kScanTile (n <= 2^24)
-    k_scan_tiles<<<n_tiles, kScanThreads, 0, s>>>(b.counts, n_rays, b.offsets, b.block_sums);
-    k_scan_top<<<1, kScanThreads, 0, s>>>(b.block_sums, n_tiles, b.offsets + n_rays);
-    k_scan_add<<<(n_rays + 255) / 256, 256, 0, s>>>(b.offsets, n_rays, b.block_sums);
-    k_compact<<<(n_rays + 7) / 8, 256, 0, s>>>(n_rays, c.max_samples, b.offsets, slots, b.ray_id, b.t);
+    k_march<<<(n_rays + 7) / 8, 256, 0, s>>>(c, occ_bits, n_rays, b.rays, b.cap_rays, b.counts, slots,
+                                             tile_totals(b, sel != nullptr));
+    launch_compact(n_rays, c.max_samples, b, slots, sel_off, sel, evaluated, s);
 }
 
 }  // namespace nm

@@ -37,4 +37,75 @@ __device__ __forceinline__ void store_ray(float* rays, uint32_t cap, uint32_t r,
     rays[kKf * cap + r] = __uint_as_float(kf);
 }
 
+// Totals of the rays' sample counts per tile of kScanTile rays, from which k_compact and
+// k_select find where a ray's samples go: all samples, the first kRenderFirst of each ray,
+// the samples a render's second pass still evaluates.  The ray generation clears them
+// (first, live: nullptr in a step), k_march and the compositing add to them.
+struct TileTotals {
+    uint32_t *all, *first, *live;
+};
+inline TileTotals tile_totals(const StepBufs& b, bool render) {
+    // a render does not use the partials of the training compositing
+    uint32_t* p = reinterpret_cast<uint32_t*>(b.partials);
+    return TileTotals{b.block_sums, render ? p : nullptr, render ? p + kCompositeMaxBlocks : nullptr};
+}
+static_assert((1u << 24) / kScanTile <= kCompositeMaxBlocks, "the totals of the largest batch fit the partials");
+
+__device__ __forceinline__ void clear_totals(const TileTotals& t, uint32_t i, uint32_t n_rays) {
+    if (i * (uint32_t)kScanTile >= n_rays || i >= n_rays) return;
+    t.all[i] = 0u;
+    if (t.first) t.first[i] = 0u;
+    if (t.live) t.live[i] = 0u;
+}
+
+// The march of one ray by one warp: retained steps to row (max_samples at most), their
+// number returned to all lanes.
+__device__ __forceinline__ uint32_t march_ray(const DevCfg& c, const uint32_t* __restrict__ bits,
+                                              const float* __restrict__ rays, uint32_t cap, uint32_t r, float* row) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const float3 o = make_float3(rays[kOx * cap + r], rays[kOy * cap + r], rays[kOz * cap + r]);
+    const float3 d = make_float3(rays[kDx * cap + r], rays[kDy * cap + r], rays[kDz * cap + r]);
+    const uint32_t max_samples = c.max_samples;
+    uint32_t i_lo, i_hi;
+    box_step_range(c, o, d, i_lo, i_hi);
+    uint32_t n = 0;
+    for (uint32_t i0 = i_lo; i0 < i_hi && n < max_samples; i0 += 32) {
+        const uint32_t i = i0 + lane;
+        bool keep = false;
+        float t = 0.f;
+        if (i < i_hi) {
+            t = sample_t(c, i);
+            const float3 x = grid_pos(c, o, d, t);
+            keep = in_box(c, x) && occupied(c, bits, x);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, keep);
+        const uint32_t pos = n + __popc(m & ((1u << lane) - 1u));
+        if (keep && pos < max_samples) row[pos] = t;
+        n += __popc(m);
+    }
+    return n < max_samples ? n : max_samples;
+}
+
+// Count n of the warp's ray r to counts, and the block's 8 rays (of one tile) to the totals.
+__device__ __forceinline__ void ray_totals(const TileTotals& t, uint32_t r, uint32_t n, uint32_t n_rays,
+                                           uint32_t* __restrict__ counts) {
+    __shared__ uint32_t cnt[8];
+    const uint32_t w = threadIdx.x >> 5;
+    if ((threadIdx.x & 31u) == 0u) {
+        cnt[w] = n;
+        if (r < n_rays) counts[r] = n;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0u) return;
+    uint32_t all = 0, first = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        all += cnt[k];
+        first += min(cnt[k], kRenderFirst);
+    }
+    if (all == 0u) return;
+    atomicAdd(t.all + r / kScanTile, all);
+    if (t.first) atomicAdd(t.first + r / kScanTile, first);
+}
+
 }  // namespace nm
