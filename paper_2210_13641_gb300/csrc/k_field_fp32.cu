@@ -2,38 +2,17 @@
 // density MLP (sigma = exp(h_0)), SH view encoding and colour MLP (sigmoid) forward
 // (steps a3-a6), and the recomputing backward pass (steps a10-a11).
 //
-// Forward: one thread per sample, weights in shared memory.  Backward: tiles of 128
-// samples whose activations are recomputed into shared memory (see there).
+// Both work on tiles of 128 samples whose activations sit in shared memory.
 #include "encoding.cuh"
 #include "internal.h"
 
 namespace nm {
 
-// Weights in shared memory, with the transposes the per-thread loops read along.
-struct SmemW {
-    float W1[kHid * kEnc];        // [j][k]
-    float W2T[kHid * kGeo];       // [j][m] = W2[m][j]
-    float W3[kHid * 32];          // [j][k]
-    float W4T[kHid * kHid];       // [j][i] = W4[i][j]
-    float W5[3 * kHid];           // [c][i]
-};
-
 // 16-byte loads, several in flight (each launch pays this once per block).
-__device__ void load_weights(SmemW& s, const float* __restrict__ mlp) {
-#pragma unroll 4
-    for (int q = threadIdx.x; q < kMlpParams / 4; q += blockDim.x) {
-        const float4 w = __ldg(reinterpret_cast<const float4*>(mlp) + q);
-        const float v[4] = {w.x, w.y, w.z, w.w};
-        const int i = 4 * q;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (i < kOffW2) s.W1[i + k] = v[k];
-            else if (i < kOffW3) s.W2T[((i - kOffW2) % kHid + k) * kGeo + (i - kOffW2) / kHid] = v[k];
-            else if (i < kOffW4) s.W3[i - kOffW3 + k] = v[k];
-            else if (i < kOffW5) s.W4T[((i - kOffW4) % kHid + k) * kHid + (i - kOffW4) / kHid] = v[k];
-            else s.W5[i - kOffW5 + k] = v[k];
-        }
-    }
+__device__ __forceinline__ void load_weights(float* W, const float* __restrict__ mlp) {
+#pragma unroll 5
+    for (int i = threadIdx.x; i < kMlpParams / 4; i += blockDim.x)
+        reinterpret_cast<float4*>(W)[i] = __ldg(reinterpret_cast<const float4*>(mlp) + i);
 }
 
 __device__ __forceinline__ float3 sample_pos(const DevCfg& c, const float* __restrict__ rays,
@@ -43,50 +22,77 @@ __device__ __forceinline__ float3 sample_pos(const DevCfg& c, const float* __res
     return grid_pos(c, o, d, t);
 }
 
-// Density MLP: y = W2 relu(W1 f).
-__device__ __forceinline__ void density_mlp(const SmemW& s, const float* f, float* y) {
+constexpr int kTile = 128;          // samples of a tile
+constexpr int kFieldThreads = 256;  // threads of a block, forward and backward
+
+// o[n][q] += sum_k W[n][k] x_q[k] for NO outputs and 4 samples (rows of ROW floats: x, 32 rows
+// on, ...) over K inputs, k ascending.
+template <int K, int NO, int ROW>
+__device__ __forceinline__ void dot_rows(const float* __restrict__ W, const float* x, float (*o)[4]) {
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+        float4 v[4];
 #pragma unroll
-    for (int m = 0; m < kGeo; ++m) y[m] = 0.f;
-#pragma unroll 2
-    for (int j = 0; j < kHid; ++j) {
-        float a = 0.f;
+        for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const float4*>(x + 32 * q * ROW + k);
 #pragma unroll
-        for (int k = 0; k < kEnc; ++k) a += s.W1[j * kEnc + k] * f[k];
-        a = fmaxf(a, 0.f);
+        for (int n = 0; n < NO; ++n) {
+            const float4 w = *reinterpret_cast<const float4*>(W + n * K + k);
 #pragma unroll
-        for (int m = 0; m < kGeo; ++m) y[m] += s.W2T[j * kGeo + m] * a;
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.x, v[q].x, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.y, v[q].y, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.z, v[q].z, o[n][q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.w, v[q].w, o[n][q]);
+        }
     }
 }
 
-// Colour MLP: rgb = sigmoid(W5 relu(W4 relu(W3 x3))).
-__device__ __forceinline__ float3 color_mlp(const SmemW& s, const float* x3) {
-    float h4[kHid];
+template <int N>
+__device__ __forceinline__ void zero(float* v) {
 #pragma unroll
-    for (int i = 0; i < kHid; ++i) h4[i] = 0.f;
-#pragma unroll 1
-    for (int j = 0; j < kHid; ++j) {
-        float a = 0.f;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) a += s.W3[j * 32 + k] * x3[k];
-        a = fmaxf(a, 0.f);
-#pragma unroll
-        for (int i = 0; i < kHid; ++i) h4[i] += s.W4T[j * kHid + i] * a;
-    }
-    float z0 = 0.f, z1 = 0.f, z2 = 0.f;
-#pragma unroll
-    for (int i = 0; i < kHid; ++i) {
-        const float h = fmaxf(h4[i], 0.f);
-        z0 += s.W5[i] * h;
-        z1 += s.W5[kHid + i] * h;
-        z2 += s.W5[2 * kHid + i] * h;
-    }
-    return make_float3(sigmoidf_(z0), sigmoidf_(z1), sigmoidf_(z2));
+    for (int k = 0; k < N; ++k) v[k] = 0.f;
 }
+
+// Output n of sample q, N of them (a multiple of 4, or 2), to the samples' rows.
+template <int N, bool RELU, int ROW>
+__device__ __forceinline__ void put(float* dst, const float (*o)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) v[n] = RELU ? fmaxf(o[n][q], 0.f) : o[n][q];
+        float* d = dst + 32 * q * ROW;
+        if constexpr (N % 4 == 0) {
+#pragma unroll
+            for (int n = 0; n < N; n += 4)
+                *reinterpret_cast<float4*>(d + n) = make_float4(v[n], v[n + 1], v[n + 2], v[n + 3]);
+        } else {
+            *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
+        }
+    }
+}
+
+// ------------------------------------------------------------------ forward
+// Tiles of 128 samples, two 256-thread blocks per SM: two threads encode each sample (half
+// the levels each), then every layer is a phase over 4 samples x 8 outputs per thread
+// (dot_rows) on activations in shared memory.  Bound by the multiply-adds (9.4 k per
+// sample: 1.2 ms for 4.87 M samples) and the loads that feed them, and the gathers.  One
+// thread per sample, all weights read again for each, took 3.31 ms there; this form
+// 2.91.
+constexpr int kFRow = 132;  // row: f[0,32) x3[32,64) h1, then h3 [64,128); h4 over f and x3
+constexpr int kFx3 = 32, kFh = 64;
+
+struct alignas(16) SmemFwd {
+    float W[kMlpParams];        // plain (out, in) layout as in the parameter buffer
+    float act[kTile * kFRow];
+};
 
 // kSel: the samples sel[0 .. *n_total) of the batch instead of 0 .. *n_total (a
 // render's passes); the encodings are not stored then.
 template <bool kSel>
-__global__ void __launch_bounds__(128) k_field_fwd_fp32(DevCfg c, const float* __restrict__ params,
+__global__ void __launch_bounds__(kFieldThreads, 2) k_field_fwd_fp32(DevCfg c, const float* __restrict__ params,
                                                         const float* __restrict__ rays, uint32_t cap,
                                                         const uint32_t* __restrict__ n_total,
                                                         const uint32_t* __restrict__ ray_id,
@@ -94,54 +100,101 @@ __global__ void __launch_bounds__(128) k_field_fwd_fp32(DevCfg c, const float* _
                                                         float4* __restrict__ sig_rgb,
                                                         float* __restrict__ feat_out,
                                                         const uint32_t* __restrict__ sel) {
-    extern __shared__ float smem_raw[];
-    SmemW& s = *reinterpret_cast<SmemW*>(smem_raw);
-    const float* mlp = params + (size_t)c.L * c.T * 2;
-    load_weights(s, mlp);
-    __syncthreads();
+    extern __shared__ __align__(16) float smem_raw[];
+    SmemFwd& s = *reinterpret_cast<SmemFwd*>(smem_raw);
     const uint32_t n = *n_total;
+    if (blockIdx.x * (uint32_t)kTile >= n) return;
+    load_weights(s.W, params + (size_t)c.L * c.T * 2);
+    const float* W5 = s.W + kOffW5;
     const float2* tables = reinterpret_cast<const float2*>(params);
-    for (uint32_t j0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n; j0 += gridDim.x * blockDim.x) {
-        // whole warps encode: lanes past the end stand at position 0
-        const uint32_t j = j0 + pair_sample(threadIdx.x & 31u);
-        const bool valid = j < n;
-        const uint32_t i = valid ? (kSel ? sel[j] : j) : 0u;
-        float3 d = make_float3(0.f, 0.f, 0.f), x = d;
-        if (valid) x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
-        float f[kEnc];
-        hash_encode(c, tables, x, f);
-        if (!valid) continue;
-        if (!kSel && feat_out) {
-            float4* fo = reinterpret_cast<float4*>(feat_out + (size_t)i * kEnc);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* const row0 = s.act + lane * kFRow;                   // layer products: samples lane, lane + 32, ...
+    const int part = tid >> 7;                                   // encoding: levels 8 part .. 8 part + 7
+    const uint32_t er = (tid & 96) + pair_sample(tid & 31);      // of this sample (whole warps)
+    float* const erow = s.act + er * kFRow;
+    float* const trow = s.act + (tid & 127) * kFRow;
+    for (uint32_t i0 = blockIdx.x * (uint32_t)kTile; i0 < n; i0 += gridDim.x * (uint32_t)kTile) {
+        {
+            const uint32_t j = i0 + er;
+            const bool valid = j < n;
+            const uint32_t i = valid ? (kSel ? sel[j] : j) : 0u;
+            float3 d = make_float3(0.f, 0.f, 0.f), x = d;
+            if (valid) x = sample_pos(c, rays, cap, ray_id[i], ts[i], d);
+            if (part) {
+                float sh[16];
+                sh16(d.x, d.y, d.z, sh);
 #pragma unroll
-            for (int k = 0; k < kEnc / 4; ++k) fo[k] = make_float4(f[4 * k], f[4 * k + 1], f[4 * k + 2], f[4 * k + 3]);
+                for (int k = 0; k < 16; k += 4)
+                    *reinterpret_cast<float4*>(erow + kFx3 + kGeo + k) = make_float4(sh[k], sh[k + 1], sh[k + 2], sh[k + 3]);
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int l = 8 * part + 2 * h;
+                float f[4] = {0.f, 0.f, 0.f, 0.f};
+                if (l < (int)c.L) encode_level(c, tables, x, l, f);
+                if (l + 1 < (int)c.L) encode_level(c, tables, x, l + 1, f + 2);
+                const float4 q = make_float4(f[0], f[1], f[2], f[3]);
+                *reinterpret_cast<float4*>(erow + 2 * l) = q;
+                if (!kSel && feat_out && valid) *reinterpret_cast<float4*>(feat_out + (size_t)i * kEnc + 2 * l) = q;
+            }
         }
-        float x3[32];
-        density_mlp(s, f, x3);
-        sh16(d.x, d.y, d.z, x3 + kGeo);
-        const float sigma = expf(fminf(x3[0], kSigmaHMax));
-        const float3 rgb = color_mlp(s, x3);
-        sig_rgb[i] = make_float4(sigma, rgb.x, rgb.y, rgb.z);
+        __syncthreads();
+        float o[8][4];
+        zero<32>(&o[0][0]);
+        dot_rows<kEnc, 8, kFRow>(s.W + kOffW1 + 8 * warp * kEnc, row0, o);
+        put<8, true, kFRow>(row0 + kFh + 8 * warp, o);
+        __syncthreads();
+        zero<8>(&o[0][0]);
+        dot_rows<kHid, 2, kFRow>(s.W + kOffW2 + 2 * warp * kHid, row0 + kFh, o);
+        put<2, false, kFRow>(row0 + kFx3 + 2 * warp, o);
+        __syncthreads();
+        const float sigma = expf(fminf(trow[kFx3], kSigmaHMax));
+        zero<32>(&o[0][0]);
+        dot_rows<32, 8, kFRow>(s.W + kOffW3 + 8 * warp * 32, row0 + kFx3, o);
+        put<8, true, kFRow>(row0 + kFh + 8 * warp, o);
+        __syncthreads();
+        zero<32>(&o[0][0]);
+        dot_rows<kHid, 8, kFRow>(s.W + kOffW4 + 8 * warp * kHid, row0 + kFh, o);
+        put<8, true, kFRow>(row0 + 8 * warp, o);
+        __syncthreads();
+        if (tid < kTile && i0 + tid < n) {
+            float z[3] = {0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int q = 0; q < kHid; q += 4) {
+                const float4 h = *reinterpret_cast<const float4*>(trow + q);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float4 w = *reinterpret_cast<const float4*>(W5 + k * kHid + q);
+                    z[k] = fmaf(w.x, h.x, z[k]);
+                    z[k] = fmaf(w.y, h.y, z[k]);
+                    z[k] = fmaf(w.z, h.z, z[k]);
+                    z[k] = fmaf(w.w, h.w, z[k]);
+                }
+            }
+            sig_rgb[kSel ? sel[i0 + tid] : i0 + tid] = make_float4(sigma, sigmoidf_(z[0]), sigmoidf_(z[1]), sigmoidf_(z[2]));
+        }
+        __syncthreads();  // the next tile overwrites the rows
     }
+}
+
+template <bool kSel>
+static void fwd_fp32(const DevCfg& c, const float* params, const uint32_t* n, const uint32_t* sel, const StepBufs& b,
+                     float* feat, int n_sm, cudaStream_t st) {
+    const int smem = (int)sizeof(SmemFwd);
+    // per call: the attribute belongs to the current device (cheap next to the kernel)
+    cudaFuncSetAttribute(k_field_fwd_fp32<kSel>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_field_fwd_fp32<kSel><<<n_sm * 2, kFieldThreads, smem, st>>>(c, params, b.rays, b.cap_rays, n, b.ray_id, b.t,
+                                                                  b.sig_rgb, feat, sel);
 }
 
 void launch_field_fwd_fp32(const DevCfg& c, const float* params, uint32_t n_rays, const StepBufs& b,
                            bool store_feat, int n_sm, cudaStream_t st) {
-    const size_t smem = sizeof(SmemW);
-    // per call: the attribute belongs to the current device (cheap next to the kernel)
-    cudaFuncSetAttribute(k_field_fwd_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    (void)n_rays;
-    k_field_fwd_fp32<false><<<n_sm * 8, 128, smem, st>>>(c, params, b.rays, b.cap_rays, b.offsets + n_rays,
-                                                        b.ray_id, b.t, b.sig_rgb, store_feat ? b.feat : nullptr,
-                                                        nullptr);
+    fwd_fp32<false>(c, params, b.offsets + n_rays, nullptr, b, store_feat ? b.feat : nullptr, n_sm, st);
 }
 
 void launch_field_fwd_fp32_sel(const DevCfg& c, const float* params, const uint32_t* sel, const uint32_t* n_sel,
                                const StepBufs& b, int n_sm, cudaStream_t st) {
-    const size_t smem = sizeof(SmemW);
-    cudaFuncSetAttribute(k_field_fwd_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_field_fwd_fp32<true><<<n_sm * 8, 128, smem, st>>>(c, params, b.rays, b.cap_rays, n_sel, b.ray_id, b.t,
-                                                       b.sig_rgb, nullptr, sel);
+    fwd_fp32<true>(c, params, n_sel, sel, b, nullptr, n_sm, st);
 }
 
 // ------------------------------------------------------------------ backward
@@ -161,8 +214,6 @@ void launch_field_fwd_fp32_sel(const DevCfg& c, const float* params, const uint3
 // and the shared-memory loads that feed them bound it.  One thread per sample with 128
 // threads per SM, whose weight-gradient products took 8 4-byte loads for 16 multiply-adds,
 // needed 14.2 ms there; this form 7.9 ms (8.6 with 2 samples x 16 outputs per thread).
-constexpr int kTile = 128;
-constexpr int kBwdThreadsF = 256;
 constexpr int kRow = 260;  // 16-byte rows; consecutive rows start 16 bytes apart modulo the banks
 // Row layout: f[0,32) h1[32,96) x3[96,128) h3[128,192) h4[192,256), then the colour
 // seeds (dL/dc, later dL/dz) and dL/dsigma (later dL/dsigma * dsigma/dh_0)
@@ -175,30 +226,6 @@ struct SmemBwd {
     float4 pos[2][kTile];         // sample positions by tile_row, by tile parity
 };
 static_assert(kMlpParams % 4 == 0, "rows of 16 bytes behind the weights");
-
-// o[n][q] += sum_k W[n][k] x_q[k] for NO outputs and 4 samples (rows x, x + 32 rows, ...)
-// over K inputs, k ascending.
-template <int K, int NO>
-__device__ __forceinline__ void dot_rows(const float* __restrict__ W, const float* x, float (*o)[4]) {
-#pragma unroll 1
-    for (int k = 0; k < K; k += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = *reinterpret_cast<const float4*>(x + 32 * q * kRow + k);
-#pragma unroll
-        for (int n = 0; n < NO; ++n) {
-            const float4 w = *reinterpret_cast<const float4*>(W + n * K + k);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.x, v[q].x, o[n][q]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.y, v[q].y, o[n][q]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.z, v[q].z, o[n][q]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) o[n][q] = fmaf(w.w, v[q].w, o[n][q]);
-        }
-    }
-}
 
 // o[k][q] += sum_n W[n][k] g_q[n] for NO consecutive k over N rows of length LD.
 template <int N, int LD, int NO>
@@ -262,31 +289,6 @@ __device__ __forceinline__ void outer_sum(const float* g, const float* x, int s0
     }
 }
 
-template <int N>
-__device__ __forceinline__ void zero(float* v) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) v[k] = 0.f;
-}
-
-// Output n of sample q, N of them (a multiple of 4, or 2), to the samples' rows.
-template <int N, bool RELU>
-__device__ __forceinline__ void put(float* dst, const float (*o)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        float v[N];
-#pragma unroll
-        for (int n = 0; n < N; ++n) v[n] = RELU ? fmaxf(o[n][q], 0.f) : o[n][q];
-        float* d = dst + 32 * q * kRow;
-        if constexpr (N % 4 == 0) {
-#pragma unroll
-            for (int n = 0; n < N; n += 4)
-                *reinterpret_cast<float4*>(d + n) = make_float4(v[n], v[n + 1], v[n + 2], v[n + 3]);
-        } else {
-            *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
-        }
-    }
-}
-
 // 8 gradients of 4 samples over their activations (masked by the ReLU branches those tell).
 __device__ __forceinline__ void put_masked(float* act, const float (*o)[4]) {
 #pragma unroll
@@ -305,7 +307,7 @@ __device__ __forceinline__ void put_masked(float* act, const float (*o)[4]) {
 // which its tile has read), and the view-direction gradient through the SH encoding into
 // pose_s[2 i + 1].
 template <bool kPose>
-__global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const float* __restrict__ params,
+__global__ void __launch_bounds__(kFieldThreads) k_field_bwd_fp32(DevCfg c, const float* __restrict__ params,
                                                           float* __restrict__ grads,
                                                           const float* __restrict__ rays, uint32_t cap,
                                                           const uint32_t* __restrict__ n_total,
@@ -319,9 +321,7 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
     const uint32_t n = *n_total;
     if (blockIdx.x * (uint32_t)kTile >= n) return;
     const float* mlp = params + (size_t)c.L * c.T * 2;
-#pragma unroll 5
-    for (int i = threadIdx.x; i < kMlpParams / 4; i += kBwdThreadsF)
-        reinterpret_cast<float4*>(s.W)[i] = __ldg(reinterpret_cast<const float4*>(mlp) + i);
+    load_weights(s.W, mlp);
     const float* W1 = s.W + kOffW1;
     const float* W2 = s.W + kOffW2;
     const float* W3 = s.W + kOffW3;
@@ -377,20 +377,20 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
         float o[8][4];
         // ---- forward recompute
         zero<32>(&o[0][0]);
-        dot_rows<kEnc, 8>(W1 + 8 * warp * kEnc, row0 + kRf, o);
-        put<8, true>(row0 + kRh1 + 8 * warp, o);
+        dot_rows<kEnc, 8, kRow>(W1 + 8 * warp * kEnc, row0 + kRf, o);
+        put<8, true, kRow>(row0 + kRh1 + 8 * warp, o);
         __syncthreads();
         zero<8>(&o[0][0]);
-        dot_rows<kHid, 2>(W2 + 2 * warp * kHid, row0 + kRh1, o);
-        put<2, false>(row0 + kRx3 + 2 * warp, o);
+        dot_rows<kHid, 2, kRow>(W2 + 2 * warp * kHid, row0 + kRh1, o);
+        put<2, false, kRow>(row0 + kRx3 + 2 * warp, o);
         __syncthreads();
         zero<32>(&o[0][0]);
-        dot_rows<32, 8>(W3 + 8 * warp * 32, row0 + kRx3, o);
-        put<8, true>(row0 + kRh3 + 8 * warp, o);
+        dot_rows<32, 8, kRow>(W3 + 8 * warp * 32, row0 + kRx3, o);
+        put<8, true, kRow>(row0 + kRh3 + 8 * warp, o);
         __syncthreads();
         zero<32>(&o[0][0]);
-        dot_rows<kHid, 8>(W4 + 8 * warp * kHid, row0 + kRh3, o);
-        put<8, true>(row0 + kRh4 + 8 * warp, o);
+        dot_rows<kHid, 8, kRow>(W4 + 8 * warp * kHid, row0 + kRh3, o);
+        put<8, true, kRow>(row0 + kRh4 + 8 * warp, o);
         __syncthreads();
         if (tid < kTile) {  // colours: dL/dz; the density's seed
             float* row = s.act + tid * kRow;
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
             for (int q = 0; q < 4; ++q) o[0][q] += row0[32 * q * kRow + kRds];
         }
         __syncthreads();
-        put<2, false>(row0 + kRx3 + 2 * warp, o);
+        put<2, false, kRow>(row0 + kRx3 + 2 * warp, o);
         __syncthreads();
         // dW2 += dy^T h1;  dA1 = (W2^T dy) [h1 > 0]
         outer_sum(s.act + kRx3 + 8 * half, s.act + kRh1 + c16, e0, 16, g2);
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
     // ---- the warps' sums meet in shared memory (act), one part after the other
     __syncthreads();
     float* dW = s.act;
-    for (int i = tid; i < kMlpParams; i += kBwdThreadsF) dW[i] = 0.f;
+    for (int i = tid; i < kMlpParams; i += kFieldThreads) dW[i] = 0.f;
     auto add = [&](int off, int ld, const float* g) {
 #pragma unroll
         for (int n = 0; n < 8; ++n)
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kBwdThreadsF) k_field_bwd_fp32(DevCfg c, const
     }
     __syncthreads();
     float* gmlp = grads + (size_t)c.L * c.T * 2;
-    for (int e = tid; e < kMlpParams; e += kBwdThreadsF) {
+    for (int e = tid; e < kMlpParams; e += kFieldThreads) {
         const float v = dW[e];
         if (v != 0.f) atomicAdd(gmlp + e, v);
     }
@@ -539,11 +539,11 @@ void launch_field_bwd_fp32(const DevCfg& c, const float* params, float* grads, u
     cudaFuncSetAttribute(k_field_bwd_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_field_bwd_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (pose)
-        k_field_bwd_fp32<true><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
+        k_field_bwd_fp32<true><<<n_sm, kFieldThreads, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
                                                                  b.offsets + n_rays, b.ray_id, b.t, b.feat, b.dsig_rgb,
                                                                  b.pose_s, b.pose_odd);
     else
-        k_field_bwd_fp32<false><<<n_sm, kBwdThreadsF, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
+        k_field_bwd_fp32<false><<<n_sm, kFieldThreads, smem, st>>>(c, params, grads, b.rays, b.cap_rays,
                                                                   b.offsets + n_rays, b.ray_id, b.t, b.feat,
                                                                   b.dsig_rgb, nullptr, nullptr);
 }
