@@ -118,15 +118,35 @@ struct MnMaj {
     static constexpr bool mn = true;
 };
 
-// D (M x N, at TMEM address d) (+)= A B over KS steps of K = 16; base4: the block's
-// shared-memory base / 16.
+// D (M x N, at TMEM address d) (+)= A B over KS steps of K = 16; a4, b4: the shared-memory
+// bases of the operands' tiles / 16.
 template <bool BF16, int M, int N, class A, class B, int KS>
-__device__ __forceinline__ void gemm(uint32_t d, uint32_t base4, bool acc) {
-    asm volatile("" : "+r"(base4), "+r"(d));  // the adds stay here: hoisted out of the tile loop they spill
+__device__ __forceinline__ void gemm(uint32_t d, uint32_t a4, uint32_t b4, bool acc) {
+    asm volatile("" : "+r"(a4), "+r"(b4), "+r"(d));  // the adds stay here: hoisted out of the tile loop they spill
 #pragma unroll
     for (int k = 0; k < KS; ++k)
         mma_f16<A::hi, B::hi, idesc_f16(M, N, BF16, A::mn, B::mn)>(
-            d, base4 + A::lo + k * (A::kstep >> 4), base4 + B::lo + k * (B::kstep >> 4), (acc || k > 0) ? 1u : 0u);
+            d, a4 + A::lo + k * (A::kstep >> 4), b4 + B::lo + k * (B::kstep >> 4), (acc || k > 0) ? 1u : 0u);
+}
+
+__device__ __forceinline__ void nb_sync(int id, int n) {
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void nb_arrive(int id, int n) {
+    asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
+
+// Whether any of the barrier's n threads passes true.
+__device__ __forceinline__ bool nb_or(int id, int n, bool v) {
+    uint32_t r;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.b32 p, %3, 0;\n"
+        "bar.red.or.pred q, %1, %2, p;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n" : "=r"(r) : "r"(id), "r"(n), "r"((uint32_t)v) : "memory");
+    return r != 0u;
 }
 
 // Makes this thread's operand writes visible to the tensor core and orders its
@@ -135,6 +155,14 @@ __device__ __forceinline__ void to_tensor() {
     fence_proxy_async();
     fence_before_sync();
     __syncthreads();
+    fence_after_sync();
+}
+
+// The same for the 128 threads of one group of the block (barrier `id`).
+__device__ __forceinline__ void to_tensor_group(int id) {
+    fence_proxy_async();
+    fence_before_sync();
+    nb_sync(id, 128);
     fence_after_sync();
 }
 
@@ -222,13 +250,22 @@ using W5M = MnMaj<kOW5, 16>;
 
 }  // namespace
 
-constexpr int kFwdSmem = kWB + kT32 + kT64;                            // 45056
+// A forward block has NG groups of 128 threads, each with its own tile buffers, TMEM columns,
+// MMA barriers and hardware barrier (1 + group), and one copy of the weight tiles.  Step and
+// render launch one block of four groups per SM: four blocks with a copy each left the L1
+// 60 KB instead of 130 (field_fwd of 19.5 M samples 3.33 ms, FWD_GROUPS_MS now; a fifth block
+// 3.84).  The grouped render switches weights between tiles and has one group per block.
+constexpr int kFwdGroups = 4;
+constexpr int kFwdTile = kT32 + kT64;
+constexpr int kFwdSmem = kWB + kFwdTile;                // one group
+constexpr int kFwdSmemN = kWB + kFwdGroups * kFwdTile;  // 118784
 
 // ------------------------------------------------------------------ forward
 // One tile of the forward: samples i0 .. min(i0 + 128, i_end) - 1; thread r of the
-// block owns sample row r, the samples of a warp in pair_sample order.  smem: the weight tiles, then tA (128 x 32: X0, X3) and
-// tB (128 x 64: H1, H3, H4; a layer's MMAs have completed before its output
-// overwrites its input).  Returns after the tile's last MMA wait.
+// group owns sample row r, the samples of a warp in pair_sample order.  smem: the weight
+// tiles, then per group tA (128 x 32: X0, X3) and tB (128 x 64: H1, H3, H4; a layer's MMAs
+// have completed before its output overwrites its input).  Returns after the tile's last
+// MMA wait.
 // kSel: row r evaluates sample sel[i0 + r] of the batch instead of i0 + r (a render's
 // passes over a subset of the samples).
 // kSplit: the levels from split_level(c) on have been gathered level by level
@@ -242,12 +279,13 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
                                          uint32_t tmem, uint64_t* bar, uint32_t& phase, bool& timed_out,
                                          const uint32_t* __restrict__ sel = nullptr,
                                          const uint32_t* __restrict__ fine = nullptr, size_t fine_stride = 0) {
-    uint8_t* tA = smem + kWB;
+    const int tid = threadIdx.x & 127, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int group = __shfl_sync(0xffffffffu, threadIdx.x >> 7, 0), bid = 1 + group;
+    uint8_t* tA = smem + kWB + group * kFwdTile;
     uint8_t* tB = tA + kT32;
     using TA = KMaj<kWB, 128>;
     using TB = KMaj<kWB + kT32, 128>;
-    const uint32_t base4 = smem_u32(smem) >> 4;
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const uint32_t b4 = smem_u32(smem) >> 4, a4 = b4 + group * (kFwdTile >> 4);
     const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
     const float inv_fs = 1.f / feat_scale;
     // which sample a row holds is free: the rows of a warp follow the encoding's pairs
@@ -290,9 +328,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
         if (!kSel && feat_out && valid) feat_out[(size_t)i * 4 + g] = q;
     }
     // layer 1: D = X0 W1^T (128 x 64)
-    to_tensor();
+    to_tensor_group(bid);
     if (warp == 0 && elect_one()) {
-        gemm<BF16, 128, 64, TA, W1K, 2>(tmem, base4, false);
+        gemm<BF16, 128, 64, TA, W1K, 2>(tmem, a4, b4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -304,9 +342,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
         store_row_at<BF16, 32, true>(tB, tid, h, v);
     }
     // layer 2: y = H1 W2^T (128 x 16)
-    to_tensor();
+    to_tensor_group(bid);
     if (warp == 0 && elect_one()) {
-        gemm<BF16, 128, 16, TB, W2K, 4>(tmem, base4, false);
+        gemm<BF16, 128, 16, TB, W2K, 4>(tmem, a4, b4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -319,9 +357,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
     }
     store_row<BF16, 32>(tA, tid, v);
     // layer 3: H3 = relu(X3 W3^T)
-    to_tensor();
+    to_tensor_group(bid);
     if (warp == 0 && elect_one()) {
-        gemm<BF16, 128, 64, TA, W3K, 2>(tmem, base4, false);
+        gemm<BF16, 128, 64, TA, W3K, 2>(tmem, a4, b4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -331,9 +369,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
         store_row_at<BF16, 32, true>(tB, tid, h, v);
     }
     // layer 4: H4 = relu(H3 W4^T)
-    to_tensor();
+    to_tensor_group(bid);
     if (warp == 0 && elect_one()) {
-        gemm<BF16, 128, 64, TB, W4K, 4>(tmem, base4, false);
+        gemm<BF16, 128, 64, TB, W4K, 4>(tmem, a4, b4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -343,9 +381,9 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
         store_row_at<BF16, 32, true>(tB, tid, h, v);
     }
     // layer 5: z = H4 W5^T (3 of 16 columns used)
-    to_tensor();
+    to_tensor_group(bid);
     if (warp == 0 && elect_one()) {
-        gemm<BF16, 128, 16, TB, W5K, 4>(tmem, base4, false);
+        gemm<BF16, 128, 16, TB, W5K, 4>(tmem, a4, b4, false);
         mma_commit(bar);
     }
     wait_mma(bar, phase, timed_out, c.wait_polls);
@@ -354,34 +392,39 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
 }
 
 // Tensor memory and barriers of a forward block: 64 TMEM columns (one 128 x 64 FP32
-// accumulator), the MMA barrier and the drain barrier.
+// accumulator), an MMA barrier and a drain barrier per group.
+template <int NG>
 __device__ __forceinline__ uint32_t fwd_block_setup(uint32_t* tslot, uint64_t* bar, uint64_t* drain_bar) {
-    if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, 64);
+    if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, 64 * NG);
     if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        mbar_init(drain_bar, 1);
+        for (int g = 0; g < NG; ++g) {
+            mbar_init(bar + g, 1);
+            mbar_init(drain_bar + g, 1);
+        }
         mbar_fence_init();
     }
     to_tensor();
     return *tslot;
 }
 
-// End of a forward block: after a timeout, drain the issued MMAs; free the TMEM.
+// End of a forward block: after a timeout, drain each group's issued MMAs; free the TMEM.
+template <int NG>
 __device__ __forceinline__ void fwd_block_finish(uint32_t tmem, uint64_t* drain_bar, bool timed_out) {
     fence_before_sync();
     const bool any_timeout = __syncthreads_or(timed_out) != 0;
     fence_after_sync();
     if (any_timeout) {
-        if (__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0) == 0 && elect_one()) drain_mma(drain_bar);
+        const uint32_t warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+        if ((warp & 3u) == 0u && elect_one()) drain_mma(drain_bar + (warp >> 2));
         fence_before_sync();
         __syncthreads();
         fence_after_sync();
     }
-    if ((threadIdx.x >> 5) == 0) tmem_dealloc(tmem, 64);
+    if ((threadIdx.x >> 5) == 0) tmem_dealloc(tmem, 64 * NG);
 }
 
 template <bool BF16, bool kSel = false, bool kSplit = false>
-__global__ void __launch_bounds__(128, 4) k_field_fwd_tc(DevCfg c, const float* __restrict__ params,
+__global__ void __launch_bounds__(128 * kFwdGroups, 1) k_field_fwd_tc(DevCfg c, const float* __restrict__ params,
                                                       const float* __restrict__ rays, uint32_t cap,
                                                       const uint32_t* __restrict__ n_total,
                                                       const uint32_t* __restrict__ ray_id,
@@ -392,27 +435,31 @@ __global__ void __launch_bounds__(128, 4) k_field_fwd_tc(DevCfg c, const float* 
                                                       const uint32_t* __restrict__ fine = nullptr,
                                                       size_t fine_stride = 0) {
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ uint64_t bar, drain_bar;
+    __shared__ uint64_t bar[kFwdGroups], drain_bar[kFwdGroups];
     __shared__ uint32_t tslot;
     const uint32_t n = *n_total;
     if (blockIdx.x * 128u >= n) return;
-    load_weight_tiles<BF16, 128>(params + (size_t)c.L * c.T * 2, smem, threadIdx.x);
-    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
+    load_weight_tiles<BF16, 128 * kFwdGroups>(params + (size_t)c.L * c.T * 2, smem, threadIdx.x);
+    const uint32_t tmem = fwd_block_setup<kFwdGroups>(&tslot, bar, drain_bar);
     const uint32_t n_tiles = (n + 127) / 128;
     const float2* tables = reinterpret_cast<const float2*>(params);
     uint32_t phase = 0;
     bool timed_out = false;
-    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const int group = __shfl_sync(0xffffffffu, threadIdx.x >> 7, 0);
+    // a group's tiles; the first of every block before the second of any
+    for (uint32_t tile = group * gridDim.x + blockIdx.x; tile < n_tiles; tile += kFwdGroups * gridDim.x) {
         const uint32_t i0 = tile * 128;
-        fwd_tile<BF16, kSel, kSplit>(c, tables, rays, cap, ray_id, ts, sig_rgb, feat_out, feat_scale, i0, n, smem, tmem,
-                                     &bar, phase, timed_out, sel, fine, fine_stride);
+        fwd_tile<BF16, kSel, kSplit>(c, tables, rays, cap, ray_id, ts, sig_rgb, feat_out, feat_scale, i0, n, smem,
+                                     tmem + 64u * group, bar + group, phase, timed_out, sel, fine, fine_stride);
         fence_before_sync();
-        if (__syncthreads_or(timed_out)) {
-            if (threadIdx.x == 0) atomicOr(err, kErrTimeout);
+        if (nb_or(1 + group, 128, timed_out)) {
+            timed_out = true;
+            if ((threadIdx.x & 127) == 0) atomicOr(err, kErrTimeout);
             break;
         }
+        fence_after_sync();
     }
-    fwd_block_finish(tmem, &drain_bar, timed_out);
+    fwd_block_finish<kFwdGroups>(tmem, drain_bar, timed_out);
 }
 
 // ------------------------------------------------------------------ level by level
@@ -520,7 +567,7 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
     __shared__ uint32_t tile0_s[kGroupMaxItems + 1];
     const uint32_t total = *n_tiles_total;
     if (blockIdx.x >= total) return;
-    const uint32_t tmem = fwd_block_setup(&tslot, &bar, &drain_bar);
+    const uint32_t tmem = fwd_block_setup<1>(&tslot, &bar, &drain_bar);
     if (threadIdx.x < n_items) tile0_s[threadIdx.x] = items[threadIdx.x].tile0;
     if (threadIdx.x == 0) tile0_s[n_items] = total;
     __syncthreads();
@@ -552,7 +599,7 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
             break;
         }
     }
-    fwd_block_finish(tmem, &drain_bar, timed_out);
+    fwd_block_finish<1>(tmem, &drain_bar, timed_out);
 }
 
 // ------------------------------------------------------------------ backward
@@ -589,21 +636,6 @@ constexpr int kXBytes = 2 * 128 * 16;       // sample positions (x, valid) of th
 constexpr int kBwdSmem = kWB + kT32 + kT64 + kT32 + kT64 + kT64 + kT16 + kDfBytes + kRowBytes + kXBytes;  // 114688
 
 namespace {
-
-__device__ __forceinline__ void nb_sync(int id, int n) {
-    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
-}
-__device__ __forceinline__ void nb_arrive(int id, int n) {
-    asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(n) : "memory");
-}
-
-// to_tensor() for the 128 threads of the MLP group only.
-__device__ __forceinline__ void to_tensor_mlp() {
-    fence_proxy_async();
-    fence_before_sync();
-    nb_sync(kBarMlp, 128);
-    fence_after_sync();
-}
 
 // ReLU branches of 32 consecutive columns in one word: bit 15 - j is column 2 j's,
 // bit 31 - j column 2 j + 1's.
@@ -759,16 +791,16 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             float v[32];
             uint32_t m1[2], m3[2], m4[2];
             // ---- forward recompute (same arithmetic as the forward kernel)
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 128, 64, X0K, W1K, 2>(tmem, base4, false);
+                gemm<BF16, 128, 64, X0K, W1K, 2>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
             relu_epilogue<BF16>(trow, tH1, r, inv_fs, m1);
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 128, 16, H1K, W2K, 4>(tmem, base4, false);
+                gemm<BF16, 128, 16, H1K, W2K, 4>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -782,16 +814,16 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
                 for (int q = kGeo; q < 32; ++q) y[q] = 0.f;
             }
             store_row_at<BF16, 32>(tX3, r, 0, y);
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 128, 64, X3K, W3K, 2>(tmem, base4, false);
+                gemm<BF16, 128, 64, X3K, W3K, 2>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
             relu_epilogue<BF16>(trow, tH3, r, 1.f, m3);
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 128, 64, H3K, W4K, 4>(tmem, base4, false);
+                gemm<BF16, 128, 64, H3K, W4K, 4>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -804,28 +836,28 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             for (int q = 3; q < 16; ++q) v[q] = 0.f;
             store_row_at<BF16, 16>(tG5, r, 0, v);
             // ---- backward: dW5^T += H4^T G5 ; dH4 = G5 W5
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 64, 16, H4M, G5M, 8>(tmem + kColW5T, base4, k > 0);
-                gemm<BF16, 128, 64, G5K, W5M, 1>(tmem, base4, false);
+                gemm<BF16, 64, 16, H4M, G5M, 8>(tmem + kColW5T, base4, base4, k > 0);
+                gemm<BF16, 128, 64, G5K, W5M, 1>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
             mask_epilogue<BF16>(trow, tH4, r, m4);                 // G4
             // dW4 += G4^T H3 ; dH3 = G4 W4
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 64, 64, H4M, H3M, 8>(tmem + kColW4, base4, k > 0);
-                gemm<BF16, 128, 64, H4K, W4M, 4>(tmem, base4, false);
+                gemm<BF16, 64, 64, H4M, H3M, 8>(tmem + kColW4, base4, base4, k > 0);
+                gemm<BF16, 128, 64, H4K, W4M, 4>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
             mask_epilogue<BF16>(trow, tH3, r, m3);                 // G3
             // dW3 += G3^T X3 ; dX3 = G3 W3
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 64, 32, H3M, X3M, 8>(tmem + kColW3, base4, k > 0);
-                gemm<BF16, 128, 32, H3K, W3M, 4>(tmem, base4, false);
+                gemm<BF16, 64, 32, H3M, X3M, 8>(tmem + kColW3, base4, base4, k > 0);
+                gemm<BF16, 128, 32, H3K, W3M, 4>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -844,19 +876,19 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
             v[0] += S * rz.w * sig_grad;                                 // dL/dh_0 += dL/dsigma * dsigma/dh_0
             store_row_at<BF16, 16>(tX3, r, 0, v);                        // G2 (columns 0..15)
             // dW2^T += H1^T G2 ; dH1 = G2 W2
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 64, 16, H1M, X3M, 8>(tmem + kColW2T, base4, k > 0);
-                gemm<BF16, 128, 64, X3K, W2M, 1>(tmem, base4, false);
+                gemm<BF16, 64, 16, H1M, X3M, 8>(tmem + kColW2T, base4, base4, k > 0);
+                gemm<BF16, 128, 64, X3K, W2M, 1>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
             mask_epilogue<BF16>(trow, tH1, r, m1);                 // G1
             // dW1 += G1^T X0 ; dF = G1 W1
-            to_tensor_mlp();
+            to_tensor_group(kBarMlp);
             if (warp == 0 && elect_one()) {
-                gemm<BF16, 64, 32, H1M, X0M, 8>(tmem + kColW1, base4, k > 0);
-                gemm<BF16, 128, 32, H1K, W1M, 4>(tmem, base4, false);
+                gemm<BF16, 64, 32, H1M, X0M, 8>(tmem + kColW1, base4, base4, k > 0);
+                gemm<BF16, 128, 32, H1K, W1M, 4>(tmem, base4, base4, false);
                 mma_commit(&bar);
             }
             wait_mma(&bar, phase, timed_out, c.wait_polls);
@@ -1012,14 +1044,14 @@ static void fwd_tc(const DevCfg& c, const float* params, uint32_t n_rays, const 
         uint32_t* fine = static_cast<uint32_t*>(fine_buffer(b));
         k_gather_levels<BF16><<<n_sm * 6, 256, 0, s>>>(c, params, b.rays, b.cap_rays, b.offsets + n_rays, b.ray_id, b.t,
                                                        fs, fine, b.cap_samples);
-        cudaFuncSetAttribute(k_field_fwd_tc<BF16, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
-        k_field_fwd_tc<BF16, false, true><<<n_sm * 4, 128, kFwdSmem, s>>>(
+        cudaFuncSetAttribute(k_field_fwd_tc<BF16, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmemN);
+        k_field_fwd_tc<BF16, false, true><<<n_sm, 128 * kFwdGroups, kFwdSmemN, s>>>(
             c, params, b.rays, b.cap_rays, b.offsets + n_rays, b.ray_id, b.t, b.sig_rgb, feat, fs, b.err, nullptr, fine,
             b.cap_samples);
         return;
     }
-    cudaFuncSetAttribute(k_field_fwd_tc<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
-    k_field_fwd_tc<BF16><<<n_sm * 4, 128, kFwdSmem, s>>>(c, params, b.rays, b.cap_rays, b.offsets + n_rays,
+    cudaFuncSetAttribute(k_field_fwd_tc<BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmemN);
+    k_field_fwd_tc<BF16><<<n_sm, 128 * kFwdGroups, kFwdSmemN, s>>>(c, params, b.rays, b.cap_rays, b.offsets + n_rays,
                                                           b.ray_id, b.t, b.sig_rgb, feat, fs, b.err);
 }
 
@@ -1056,9 +1088,9 @@ static void bwd_tc(const DevCfg& c, const float* params, float* grads, uint32_t 
 template <bool BF16>
 static void fwd_tc_sel(const DevCfg& c, const float* params, const uint32_t* sel, const uint32_t* n_sel,
                        const StepBufs& b, int n_sm, cudaStream_t s) {
-    cudaFuncSetAttribute(k_field_fwd_tc<BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem);
+    cudaFuncSetAttribute(k_field_fwd_tc<BF16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmemN);
     const float fs = BF16 ? 1.f : 256.f;
-    k_field_fwd_tc<BF16, true><<<n_sm * 4, 128, kFwdSmem, s>>>(c, params, b.rays, b.cap_rays, n_sel, b.ray_id, b.t,
+    k_field_fwd_tc<BF16, true><<<n_sm, 128 * kFwdGroups, kFwdSmemN, s>>>(c, params, b.rays, b.cap_rays, n_sel, b.ray_id, b.t,
                                                                 b.sig_rgb, nullptr, fs, b.err, sel);
 }
 
