@@ -252,13 +252,16 @@ using W5M = MnMaj<kOW5, 16>;
 
 // A forward block has NG groups of 128 threads, each with its own tile buffers, TMEM columns,
 // MMA barriers and hardware barrier (1 + group), and one copy of the weight tiles.  Step and
-// render launch one block of four groups per SM: four blocks with a copy each left the L1
-// 60 KB instead of 130 (field_fwd of 19.5 M samples 3.33 ms, FWD_GROUPS_MS now; a fifth block
-// 3.84).  The grouped render switches weights between tiles and has one group per block.
-constexpr int kFwdGroups = 4;
+// render launch one block of six groups per SM, which leaves the L1 about 90 KB for the
+// gathers: field_fwd of 19.5 M samples 2.82 ms (five groups 2.87, four 3.09, three 3.63).  Four blocks
+// with a copy of the weights each left 60 KB and took 3.33, five 3.84.  The grouped render
+// switches weights between tiles and has one group per block.
+constexpr int kFwdGroups = 6;
 constexpr int kFwdTile = kT32 + kT64;
 constexpr int kFwdSmem = kWB + kFwdTile;                // one group
-constexpr int kFwdSmemN = kWB + kFwdGroups * kFwdTile;  // 118784
+constexpr int kFwdSmemN = kWB + kFwdGroups * kFwdTile;  // 167936
+// TMEM columns of NG groups: an allocation is a power of two
+constexpr uint32_t fwd_cols(int NG) { return NG == 1 ? 64u : NG == 2 ? 128u : NG <= 4 ? 256u : 512u; }
 
 // ------------------------------------------------------------------ forward
 // One tile of the forward: samples i0 .. min(i0 + 128, i_end) - 1; thread r of the
@@ -395,7 +398,7 @@ __device__ __forceinline__ void fwd_tile(const DevCfg& c, const float2* __restri
 // accumulator), an MMA barrier and a drain barrier per group.
 template <int NG>
 __device__ __forceinline__ uint32_t fwd_block_setup(uint32_t* tslot, uint64_t* bar, uint64_t* drain_bar) {
-    if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, 64 * NG);
+    if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, fwd_cols(NG));
     if (threadIdx.x == 0) {
         for (int g = 0; g < NG; ++g) {
             mbar_init(bar + g, 1);
@@ -420,7 +423,7 @@ __device__ __forceinline__ void fwd_block_finish(uint32_t tmem, uint64_t* drain_
         __syncthreads();
         fence_after_sync();
     }
-    if ((threadIdx.x >> 5) == 0) tmem_dealloc(tmem, 64 * NG);
+    if ((threadIdx.x >> 5) == 0) tmem_dealloc(tmem, fwd_cols(NG));
 }
 
 template <bool BF16, bool kSel = false, bool kSplit = false>

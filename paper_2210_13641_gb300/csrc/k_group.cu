@@ -6,8 +6,8 @@
 // ray casting, march with the scene's box and occupancy, count scan and compaction,
 // the tensor-core field forward, compositing and the output write - with each ray
 // taking its scene's configuration, parameters and bitfield from its piece.  The
-// field forward runs over 128-sample tiles that never mix two pieces, so every sample
-// goes through exactly the arithmetic of a render of its view alone; like map_render,
+// field forward of a batch of several scenes runs over 128-sample tiles that never mix two
+// pieces, and every sample goes through exactly the arithmetic of a render of its view alone; like map_render,
 // the field is evaluated in two passes when a threshold is set (the first
 // kRenderFirst samples of every ray, then the rays still above it), and the grouped
 // result equals the single-view render bit for bit.
@@ -178,21 +178,35 @@ int render_group(const GroupView* views, uint32_t n, bool bf16, GroupBufs& g, in
         k_group_march<<<(rays + 7) / 8, 256, 0, s>>>(g.items, rays, b.rays, b.cap_rays, b.counts, slots,
                                                      g.row_stride, tile_totals(b, true));
         launch_compact(rays, g.row_stride, b, slots, g.sel_off, two_pass ? g.sel : nullptr, render_eval_counter(b), s);
+        // pieces of one scene need no tile table and no switch of weights: their samples go
+        // through the single view's forward, whose groups share the weights (HD, 640x360 and
+        // 160x120 views of three maps: 11.2 -> GROUP_ONE_MS ms)
+        bool one_scene = true;
+        for (uint32_t k = 1; k < n_items; ++k) one_scene &= its.it[k].params == its.it[0].params;
+        const DevCfg& c0 = its.it[0].c;
         if (!two_pass) {
-            k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, b.offsets, g.n_tiles);
-            launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s);
+            if (one_scene) {
+                launch_field_fwd_tc(c0, its.it[0].params, rays, b, false, bf16, n_sm, s);
+            } else {
+                k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, b.offsets, g.n_tiles);
+                launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s);
+            }
             launch_composite_group(g.items, rays, b, s);
-            if (launches) *launches += 8;  // items, rays, march, compaction, tiles, field, composite, write
+            if (launches) *launches += one_scene ? 7 : 8;  // items, rays, march, compaction, (tiles), field, composite, write
         } else {
             // as map_render: the field for the first kRenderFirst samples of every ray,
             // then for the rays still above their threshold (pieces index the selection)
             for (int pass = 1; pass <= 2; ++pass) {
                 if (pass == 2) launch_select(rays, b, b.counts, g.sel_off, g.sel, render_eval_counter(b), s);
-                k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, g.sel_off, g.n_tiles);
-                launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s, g.sel);
+                if (one_scene) {
+                    launch_field_fwd_tc_sel(c0, its.it[0].params, g.sel, g.sel_off + rays, b, bf16, n_sm, s);
+                } else {
+                    k_group_tiles<<<1, 32, 0, s>>>(g.items, n_items, g.sel_off, g.n_tiles);
+                    launch_group_fwd_tc(g.items, n_items, g.n_tiles, b, bf16, n_sm, s, g.sel);
+                }
                 launch_composite_group(g.items, rays, b, s, pass, b.counts);
             }
-            if (launches) *launches += 12;
+            if (launches) *launches += one_scene ? 10 : 12;
         }
         launch_write_group(g.items, rays, b, s);
         if (cudaGetLastError() != cudaSuccess) return MAP_ECUDA;
