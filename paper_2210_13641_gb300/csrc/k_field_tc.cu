@@ -611,8 +611,8 @@ __global__ void __launch_bounds__(128, 4) k_group_fwd_tc(const GroupItem* __rest
 // (the "IO" group, thread 128 + r serves row r) load each tile's inputs one tile
 // ahead; warps 4-11 (IO and the "SC" group) scatter each finished tile's encoding
 // gradient into the tables, by level (scatter_tile), while the MLP group runs the next
-// tile.  For 19.5 M samples the chain alone takes 2.3 ms and the scatter alone 4.1 (of
-// 4.3 together): the scatter sets the pace, by its issue slots and its reductions.
+// tile.  For 19.5 M samples the chain alone takes 2.3 ms and the scatter alone 4.3,
+// as long as both together: the scatter sets the pace, by its issue slots and its reductions.
 // Registers are split with setmaxnreg: the block is launched with 80 per thread (two
 // blocks of 384 threads per SM), the MLP group takes 96 (its epilogues hold 16 columns
 // at a time), the IO group 80 and the SC group 64, which is 240 = 3 x 80; 104 / 80 / 56

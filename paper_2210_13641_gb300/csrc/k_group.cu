@@ -180,7 +180,7 @@ int render_group(const GroupView* views, uint32_t n, bool bf16, GroupBufs& g, in
         launch_compact(rays, g.row_stride, b, slots, g.sel_off, two_pass ? g.sel : nullptr, render_eval_counter(b), s);
         // pieces of one scene need no tile table and no switch of weights: their samples go
         // through the single view's forward, whose groups share the weights (HD, 640x360 and
-        // 160x120 views of three maps: 11.2 -> GROUP_ONE_MS ms)
+        // 160x120 views of three maps: 14.4 -> 12.4 ms, with that forward's six groups)
         bool one_scene = true;
         for (uint32_t k = 1; k < n_items; ++k) one_scene &= its.it[k].params == its.it[0].params;
         const DevCfg& c0 = its.it[0].c;
