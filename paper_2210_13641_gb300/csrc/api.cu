@@ -152,7 +152,7 @@ int ensure_step_bufs(map_scene* h, uint32_t n_rays) {
     StepBufs b{};
     const uint32_t cap = std::max<uint32_t>(n_rays, 1024);
     const uint64_t cs = (uint64_t)cap * h->cfg.max_samples;
-    const uint32_t n_tiles = (cap + kScanTile - 1) / kScanTile;
+    const uint32_t n_tiles = ray_tiles(cap);
     struct Req { void** p; size_t bytes; };
     std::vector<Req> reqs = {
         {(void**)&b.rays, sizeof(float) * kRayPlanes * cap},

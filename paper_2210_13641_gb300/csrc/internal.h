@@ -37,6 +37,10 @@ constexpr uint32_t kCompositeMaxBlocks = 4096;
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;
 constexpr int kScanTile = kScanThreads * kScanPer;
+// Tiles of a batch of n_rays rays (at most 2^24).
+__host__ __device__ constexpr uint32_t ray_tiles(uint32_t n_rays) {
+    return (n_rays + (uint32_t)kScanTile - 1u) / (uint32_t)kScanTile;
+}
 
 struct StepBufs {
     float* rays;            // [kRayPlanes][cap_rays]

@@ -88,7 +88,7 @@ __global__ void k_group_tiles(GroupItem* __restrict__ items, uint32_t n_items, c
 int group_bufs_alloc(GroupBufs& g, uint32_t cap_rays, uint32_t row_stride) {
     StepBufs b{};
     const uint64_t cs = (uint64_t)cap_rays * row_stride;
-    const uint32_t n_tiles = (cap_rays + kScanTile - 1) / kScanTile;
+    const uint32_t n_tiles = ray_tiles(cap_rays);
     struct Req {
         void** p;
         size_t bytes;

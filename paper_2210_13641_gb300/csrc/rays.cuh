@@ -49,10 +49,14 @@ inline TileTotals tile_totals(const StepBufs& b, bool render) {
     uint32_t* p = reinterpret_cast<uint32_t*>(b.partials);
     return TileTotals{b.block_sums, render ? p : nullptr, render ? p + kCompositeMaxBlocks : nullptr};
 }
-static_assert((1u << 24) / kScanTile <= kCompositeMaxBlocks, "the totals of the largest batch fit the partials");
+static_assert(ray_tiles(1u << 24) <= kCompositeMaxBlocks, "the totals of the largest batch fit the partials");
+
+// Whether thread i of a batch's ray generation clears the totals of tile i.  The tiles are
+// counted, not i * kScanTile compared with n_rays: that product wraps from thread 2^20 on.
+__host__ __device__ __forceinline__ bool clears_tile(uint32_t i, uint32_t n_rays) { return i < ray_tiles(n_rays); }
 
 __device__ __forceinline__ void clear_totals(const TileTotals& t, uint32_t i, uint32_t n_rays) {
-    if (i * (uint32_t)kScanTile >= n_rays || i >= n_rays) return;
+    if (!clears_tile(i, n_rays)) return;
     t.all[i] = 0u;
     if (t.first) t.first[i] = 0u;
     if (t.live) t.live[i] = 0u;
