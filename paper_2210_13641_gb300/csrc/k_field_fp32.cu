@@ -207,13 +207,18 @@ void launch_field_fwd_fp32_sel(const DevCfg& c, const float* params, const uint3
 //    The recompute sums in the forward kernel's order, so its ReLU branches are the
 //    forward's, bit for bit;
 //  - weight gradients: a thread owns 8 rows and 4 columns of each weight matrix for a part
-//    of the samples (3 16-byte loads for 32 multiply-adds); its sums stay in registers over
-//    all tiles of the block and meet in shared memory at its end;
+//    of the samples (3 16-byte loads for 32 multiply-adds).  A matrix has 2, 4 or 8 such
+//    parts, of 64, 32 or 16 samples of a tile; in turn, one part per tile adds its registers
+//    to the block's sums in shared memory and clears them.  So no FP32 sum runs over more
+//    than 128 products, nor over more than the block's tiles after that, and no two parts
+//    meet at an entry.  Registers kept over all tiles took 7.92 instead of 8.05 ms, but a
+//    flat sum over the 13.8 k equal products of a thread's 215 tiles is off by 1e-4 of
+//    itself (this one: 2e-6);
 //  - the encoding gradient goes through shared memory to the tile scatter.
 // The multiply-adds (28 k per sample: 3.6 ms for 4.87 M samples at the FP32 cores' rate)
 // and the shared-memory loads that feed them bound it.  One thread per sample with 128
 // threads per SM, whose weight-gradient products took 8 4-byte loads for 16 multiply-adds,
-// needed 14.2 ms there; this form 7.9 ms (8.6 with 2 samples x 16 outputs per thread).
+// needed 14.2 ms there; this form 8.05 ms (with 2 samples x 16 outputs per thread it took 0.7 more).
 constexpr int kRow = 260;  // 16-byte rows; consecutive rows start 16 bytes apart modulo the banks
 // Row layout: f[0,32) h1[32,96) x3[96,128) h3[128,192) h4[192,256), then the colour
 // seeds (dL/dc, later dL/dz) and dL/dsigma (later dL/dsigma * dsigma/dh_0)
@@ -221,7 +226,8 @@ constexpr int kRf = 0, kRh1 = 32, kRx3 = 96, kRh3 = 128, kRh4 = 192, kRdz = 256,
 
 struct SmemBwd {
     float W[kMlpParams];          // plain (out, in) layout as in the parameter buffer
-    float act[kTile * kRow];      // at the end: the block's weight gradients
+    float dW[kMlpParams];         // the block's weight gradients
+    float act[kTile * kRow];
     float2 df[kTile * 16];        // dL/dfeat by tile_df
     float4 pos[2][kTile];         // sample positions by tile_row, by tile parity
 };
@@ -335,16 +341,44 @@ __global__ void __launch_bounds__(kFieldThreads) k_field_bwd_fp32(DevCfg c, cons
     // warp each other samples or rows), 32 columns 8 lanes.
     const int c16 = 4 * (lane & 15), c8 = 4 * (lane & 7), half = lane >> 4, quart = lane >> 3, e0 = warp * 16;
     const uint32_t level = scatter_level(c, tid);
+    for (int i = tid; i < kMlpParams; i += kFieldThreads) s.dW[i] = 0.f;  // added to many barriers later
     float g1[32], g2[32], g3[32], g4[32], g5[6];
     zero<32>(g1);
     zero<32>(g2);
     zero<32>(g3);
     zero<32>(g4);
     zero<6>(g5);
+    auto add = [&](int off, int ld, float* g) {
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+            float4* p = reinterpret_cast<float4*>(s.dW + off + n * ld);
+            const float4 v = *p;
+            *p = make_float4(v.x + g[4 * n], v.y + g[4 * n + 1], v.z + g[4 * n + 2], v.w + g[4 * n + 3]);
+        }
+        zero<32>(g);
+    };
+    // the sums of part p4 (of W4), p3 (W3, W1) and p2 (W2, W5) into dW
+    auto add_part = [&](int p4, int p3, int p2) {
+        if (half == p4) add(kOffW4 + 8 * warp * kHid + c16, kHid, g4);
+        if (quart == p3) {
+            add(kOffW3 + 8 * warp * 32 + c8, 32, g3);
+            add(kOffW1 + 8 * warp * kEnc + c8, kEnc, g1);
+        }
+        if (warp == p2) {
+            add(kOffW2 + 8 * half * kHid + c16, kHid, g2);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                float2* p = reinterpret_cast<float2*>(s.dW + kOffW5 + k * kHid + 2 * lane);
+                const float2 v = *p;
+                *p = make_float2(v.x + g5[2 * k], v.y + g5[2 * k + 1]);
+            }
+            zero<6>(g5);
+        }
+    };
     const uint32_t n_tiles = (n + kTile - 1) / kTile;
-    uint32_t parity = 0;
-    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, parity ^= 1u) {
-        const uint32_t i0 = tile * kTile;
+    int turn = 0;  // the block's tiles, counted
+    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++turn) {
+        const uint32_t i0 = tile * kTile, parity = turn & 1;
         {   // inputs: two threads per sample
             const int r = tid & 127, part = tid >> 7;
             const uint32_t i = i0 + r;
@@ -484,6 +518,7 @@ __global__ void __launch_bounds__(kFieldThreads) k_field_bwd_fp32(DevCfg c, cons
             s.df[tile_df<16>(lane + 32 * q, 2 * warp + 1)] = make_float2(o[2][q], o[3][q]);
         }
         __syncthreads();
+        add_part(turn & 1, turn & 3, turn & 7);  // the next part's turn is behind the next tile's barriers
         scatter_tile<16>(c, gtables, tid, level, c.L, s.pos[parity], s.df, n - i0);
         if (kPose) {  // dL/dp: warps 0-3 the even levels, 4-7 the odd ones
             const int odd = tid >> 7;
@@ -498,36 +533,15 @@ __global__ void __launch_bounds__(kFieldThreads) k_field_bwd_fp32(DevCfg c, cons
         // the next tile's inputs go to rows that nobody reads any more, and to the other
         // position buffer; dL/dfeat is written again many barriers later
     }
-    // ---- the warps' sums meet in shared memory (act), one part after the other
-    __syncthreads();
-    float* dW = s.act;
-    for (int i = tid; i < kMlpParams; i += kFieldThreads) dW[i] = 0.f;
-    auto add = [&](int off, int ld, const float* g) {
-#pragma unroll
-        for (int n = 0; n < 8; ++n)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) dW[off + n * ld + k] += g[4 * n + k];
-    };
+    // ---- what each part has left, one after the other
     for (int part = 0; part < 8; ++part) {
         __syncthreads();
-        if (half == part) add(kOffW4 + 8 * warp * kHid + c16, kHid, g4);
-        if (quart == part) {
-            add(kOffW3 + 8 * warp * 32 + c8, 32, g3);
-            add(kOffW1 + 8 * warp * kEnc + c8, kEnc, g1);
-        }
-        if (warp == part) {
-            add(kOffW2 + 8 * half * kHid + c16, kHid, g2);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                dW[kOffW5 + k * kHid + 2 * lane] += g5[2 * k];
-                dW[kOffW5 + k * kHid + 2 * lane + 1] += g5[2 * k + 1];
-            }
-        }
+        add_part(part, part, part);
     }
     __syncthreads();
     float* gmlp = grads + (size_t)c.L * c.T * 2;
     for (int e = tid; e < kMlpParams; e += kFieldThreads) {
-        const float v = dW[e];
+        const float v = s.dW[e];
         if (v != 0.f) atomicAdd(gmlp + e, v);
     }
 }
