@@ -120,7 +120,7 @@ __device__ __forceinline__ void hash_encode(const DevCfg& c, const float2* __res
 // vertices in one instruction, which share a 32-byte sector 3 times in 4.
 // Per sample this issues 48.4 reductions in 33.3 sectors on the room workload's rays
 // (counted on the host), against 61.4 in 52.2 for sums over runs of equal cells within
-// a warp, and needs no shuffle at all: the backward of 19.5 M samples takes 4.28 ms
+// a warp, and needs no shuffle at all: the backward of 19.5 M samples takes 4.29 ms
 // instead of 6.74.  It runs at 0.6 of the issue rate, with the integer pipe at 0.57.
 // Walks of G = 16 samples: 8 groups and 2 parities per level, two levels per warp.  With at
 // most 8 levels to scatter (G = 8): 16 groups of 8 samples, one level per warp.
@@ -183,10 +183,11 @@ __device__ __forceinline__ void flush_if_ne(float2* p, float2& v, uint32_t a, ui
 // A vertex that leaves is told by its slot: two vertices with one slot share an entry.
 // Cells are kept as the bits of 2^23 + c: the bias, a multiple of 2^24 once multiplied,
 // vanishes under the slot mask (at most 2^24 entries).  Of an axis' two vertices one is
-// odd (O): with d = q - O the trilinear weights are 1 - |d| (odd) and |d| (even), for
-// either order of the two.  Beyond the last cell (kUnit = false: a box that reaches past
-// the unit cube, whose samples extrapolate from that cell) d takes its sign from the
-// order instead.
+// odd and one even; the trilinear weight of either is q's distance from the other, for
+// either order of the two.  (1 - |q - odd| for the odd one would save an add, but in the
+// first cell it is rounded to 2^-24 where q itself is the weight: 4.27 for 4.29 ms.)  Beyond the last cell
+// (kUnit = false: a box that reaches past the unit cube, whose samples extrapolate from that
+// cell) the distance takes its sign from the order instead.
 template <int kMode, bool kUnit>
 __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __restrict__ gtab, uint32_t mask,
                                              const float4* pos, const float2* df, uint32_t n) {
@@ -194,7 +195,6 @@ __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __res
     const uint32_t np = 1u - s.p;
     pos += s.r0;
     df += s.rd;
-    const float sx = s.p ? -1.f : 1.f, tx = s.p ? 1.f : 0.f;
     uint32_t held[4];                                     // slots by parity, [2 z + y]
     float2 acc[4];
 #pragma unroll
@@ -211,16 +211,18 @@ __device__ __forceinline__ void scatter_walk(const ScatterRole& s, float2* __res
         const uint32_t cx = __float_as_uint(__fadd_rd(fminf(qx, top), 8388608.f));
         const uint32_t cy = __float_as_uint(__fadd_rd(fminf(qy, top), 8388608.f));
         const uint32_t cz = __float_as_uint(__fadd_rd(fminf(qz, top), 8388608.f));
-        auto dist = [](float qa, uint32_t ca) {
-            const float d = fsub(qa, fsub(__uint_as_float(ca | 1u), 8388608.f));
-            return kUnit ? fabsf(d) : ((ca & 1u) ? d : -d);
+        // weight of the vertex whose other one is v (as bits); neg: that one is the upper
+        auto weight = [](float qa, uint32_t v, bool neg) {
+            const float d = fsub(qa, fsub(__uint_as_float(v), 8388608.f));
+            return kUnit ? fabsf(d) : (neg ? -d : d);
         };
-        const float dx = dist(qx, cx), dy = dist(qy, cy), dz = dist(qz, cz);
-        const uint32_t X = ((cx + np) & ~1u) | s.p;
-        const uint32_t A[2] = {((cy + 1u) & ~1u) * s.m1, (cy | 1u) * s.m1};
-        const uint32_t B[2] = {((cz + 1u) & ~1u) * s.m2, (cz | 1u) * s.m2};
-        const float fx = fmaf(sx, dx, tx);
-        const float fy[2] = {dy, 1.f - dy}, fz[2] = {dz, 1.f - dz};
+        const uint32_t X = ((cx + np) & ~1u) | s.p, xo = ((cx + s.p) & ~1u) | np;
+        const uint32_t ye = (cy + 1u) & ~1u, yo = cy | 1u, ze = (cz + 1u) & ~1u, zo = cz | 1u;
+        const uint32_t A[2] = {ye * s.m1, yo * s.m1};
+        const uint32_t B[2] = {ze * s.m2, zo * s.m2};
+        const float fx = weight(qx, xo, (cx & 1u) == s.p);
+        const float fy[2] = {weight(qy, yo, !(cy & 1u)), weight(qy, ye, cy & 1u)};
+        const float fz[2] = {weight(qz, zo, !(cz & 1u)), weight(qz, ze, cz & 1u)};
         uint32_t slot[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
