@@ -573,18 +573,19 @@ def algorithmic_bytes(cfg, n_samples, n_params):
 # the digest of the files below must match.
 NCU_TRAFFIC = {
     "sources": ["k_field_tc.cu", "encoding.cuh", "common.cuh", "tc_ptx.cuh"],
-    "sha256": "8cda8a221f64f41166e3f746ed2e7eddc0dd1370d5121e3a37c1c0f22d75b571",
+    "sha256": "a9eff84e7ac9e83799750b0bbd9f2f62c58eb91a69049f11e34188b87155d8f5",
     "samples": 15869619,
-    "field_fwd": 296292352 + 1241936896,
-    "field_bwd": 1719506688 + 98251008,
+    "field_fwd": 301837312 + 1242142720,
+    "field_bwd": 1714499840 + 25802240,
     # sm__pipe_tensor_cycles_active.avg.pct_of_peak_sustained_elapsed and
     # lts__throughput.avg.pct_of_peak_sustained_elapsed of one launch on the 32768-ray case
-    "tensor_pipe": {"field_fwd": 0.0395, "field_bwd": 0.0874},
-    "lts_throughput": {"field_fwd": 0.3192, "field_bwd": 0.5789},
+    "tensor_pipe": {"field_fwd": 0.0490, "field_bwd": 0.1367},
+    "lts_throughput": {"field_fwd": 0.3681, "field_bwd": 0.5241},
     # l1tex__data_pipe_lsu_wavefronts.sum.pct_of_peak_sustained_elapsed of the same launches: the
     # pipe that carries the gathers' and reductions' per-lane traffic, the shuffles and the
-    # shared-memory operand stores (the field kernels' binding unit at this workload)
-    "l1_data_pipe": {"field_fwd": 0.7273, "field_bwd": 0.6682},
+    # shared-memory operand stores (the forward's binding unit at this workload; the backward's
+    # scatter also takes 0.62 of the issue slots and 0.76 of the L2's reduction rate)
+    "l1_data_pipe": {"field_fwd": 0.7879, "field_bwd": 0.6496},
 }
 
 
@@ -621,14 +622,47 @@ def l2_ceilings(cfg):
     return _L2[key]
 
 
-def roofline(cfg, prof, n_samples, n_params, precision):
+def table_reductions(cfg, kfs, bits, rays=1024, seed=2000, walk=16):
+    """8-byte table reductions, and the 32-byte sectors they touch, that the backward's
+    scatter issues per sample, counted on the host over a batch of `rays` rays: walks of
+    `walk` consecutive samples hold each level's vertices by the parity of their
+    coordinates and reduce a vertex when the next sample's differs; the two x-adjacent
+    vertices of a walk that leave together share an instruction, and mostly a sector."""
+    import numpy as np
+    import oracle
+    slot, u, v = oracle.draw_rays(seed, 0, rays, [(k.W, k.H) for k in kfs])
+    o, d = oracle.cast_rays_f32(np.stack([kfs[j].c2w for j in slot]), np.stack([kfs[j].K for j in slot]), u, v)
+    x = oracle.march(cfg, o, d, bits)[3]
+    x = x[:len(x) // walk * walk]
+    reds = sectors = 0
+    for N in oracle.level_resolutions(cfg):
+        c = oracle.grid_cell_f32(x, N)[0].reshape(-1, walk, 3)
+        ends = {}
+        for k in range(8):
+            vert = np.stack([(c[..., a] | 1) if (k >> a) & 1 else (c[..., a] + (c[..., a] & 1)) for a in range(3)], -1)
+            s = oracle.vertex_index(vert, N, 1 << cfg.log2_table)
+            e = np.ones(s.shape, bool)
+            e[:, :-1] = s[:, 1:] != s[:, :-1]
+            reds += int(e.sum())
+            if k & 1:
+                e0, s0 = ends[k - 1]
+                sectors += int(e.sum()) + int(e0.sum()) - int((e & e0 & (s >> 2 == s0 >> 2)).sum())
+            else:
+                ends[k] = e, s
+    return reds / len(x), sectors / len(x)
+
+
+def roofline(cfg, prof, n_samples, n_params, precision, reductions):
     """Roofline of the step's dominant kernel.  The tables (64 MB at the room
     workload) stay in the L2, so the table traffic's bound is the L2: the forward's
     gathers are set against the L2's streaming read bandwidth, the backward's
     reductions against its streaming reduction bandwidth (both measured here over a
-    buffer the size of the tables); achieved = the table's algorithmic bytes
-    (8 corners x L levels x F features x 4 B per sample, read or reduced) / the
-    kernel's CUDA-event time.  The per-sample streams (ray data, the stored encoding,
+    buffer the size of the tables); achieved = the table's bytes / the kernel's
+    CUDA-event time: 8 corners x L levels x F features x 4 B per sample read by the
+    forward; 8 B for each reduction that the backward issues (`reductions` =
+    table_reductions(): it sums the samples of a walk first), and beside them the
+    32-byte sectors those touch, against the sectors of the streaming reductions, as
+    the L2 takes reductions by the sector.  The per-sample streams (ray data, the stored encoding,
     colours and their gradients) go to HBM; the HBM line reports the ncu DRAM bytes
     of the kernel against the measured copy bandwidth."""
     peaks = measured_peaks()
@@ -637,10 +671,10 @@ def roofline(cfg, prof, n_samples, n_params, precision):
     cand = {k: prof[k]["ms"] / max(prof[k]["count"], 1) for k in ("field_fwd", "field_bwd", "adam")}
     dom = max(cand, key=cand.get)
     l2 = l2_ceilings(cfg)
-    table_bytes = n_samples * 8 * cfg.n_levels * cfg.n_features * 4
+    per_sample = {"field_fwd": 8 * cfg.n_levels * cfg.n_features * 4, "field_bwd": 8 * reductions[0]}
     kernels = {}
     for k, peak_key in (("field_fwd", "stream_read_gbs"), ("field_bwd", "stream_reduce_gbs")):
-        ach = table_bytes / (cand[k] / 1e3) / 1e9
+        ach = n_samples * per_sample[k] / (cand[k] / 1e3) / 1e9
         tr = measured_traffic(k, precision, n_samples)
         cur = precision == "fp16" and kernel_sources_digest() == NCU_TRAFFIC["sha256"]
         lts = NCU_TRAFFIC["lts_throughput"][k] if cur else None
@@ -651,13 +685,17 @@ def roofline(cfg, prof, n_samples, n_params, precision):
                       "frac_of_random_ceiling": ach / l2["random_read_gbs" if k == "field_fwd" else "random_reduce_gbs"],
                       "hbm": {"traffic": tr, "achieved": None if tr is None else tr / (cand[k] / 1e3) / 1e9,
                               "peak": hbm, "frac": None if tr is None else tr / (cand[k] / 1e3) / 1e9 / hbm}}
+    sectors = n_samples * reductions[1] / (cand["field_bwd"] / 1e3) / 1e9
+    kernels["field_bwd"]["reductions"] = {
+        "per_sample": reductions[0], "sectors_per_sample": reductions[1], "gsectors_s": sectors,
+        "peak_gsectors_s": l2["stream_reduce_gbs"] / 32, "frac": sectors / (l2["stream_reduce_gbs"] / 32)}
     adam_gbs = ab["adam"] / (cand["adam"] / 1e3) / 1e9
     kernels["adam"] = {"bound": "hbm", "achieved": adam_gbs, "peak": hbm, "unit": "GB/s", "frac": adam_gbs / hbm,
                        "ms": cand["adam"]}
     d = kernels[dom]
     roof = {"kernel": dom, "bound": d["bound"], "achieved": d["achieved"], "peak": d["peak"], "unit": "GB/s",
             "frac": d["frac"], "traffic": measured_traffic(dom, precision, n_samples),
-            "bytes_per_sample": 8 * cfg.n_levels * cfg.n_features * 4,
+            "bytes_per_sample": per_sample.get(dom),
             "peak_source": ("L2 streaming " + ("reductions" if dom == "field_bwd" else "reads") +
                             " over a buffer the size of the tables, measured in this run" if dom != "adam"
                             else ("measured" if "hbm_gbs" in peaks else "fallback") + " HBM copy bandwidth"),
@@ -807,7 +845,7 @@ def main():
     value = replica_throughput(n * args.steps, world, ms / 1e3)
 
     # ---------------- roofline of the dominant kernel (phase times inside the timed region)
-    roof = roofline(cfg, prof, n_samples, m.n_params, args.precision)
+    roof = roofline(cfg, prof, n_samples, m.n_params, args.precision, table_reductions(cfg, kfs, bits))
 
     # ---------------- end to end: keyframe upload from pinned host memory + step + loss read
     pinned = []

@@ -17,8 +17,9 @@ __device__ __forceinline__ float corner_weight(int k, float wx, float wy, float 
 // and 16 + i (encode_level's loads then cover 16 consecutive samples each).
 __device__ __forceinline__ uint32_t pair_sample(uint32_t lane) { return (lane >> 1) + 16u * (lane & 1u); }
 
-// Table values around grid position x at level l; called by all 32 lanes, whose
-// positions follow pair_sample.  tables: [L][T] float2.  The gathers are bound by the
+// Table values around grid position x at level l, the 4 (y, z) pairs of this lane's corners
+// (lower and upper in x), and the offsets w; called by all 32 lanes, whose positions follow
+// pair_sample.  tables: [L][T] float2.  The gathers are bound by the
 // 128-byte lines their instructions touch in the L1 (39.5 wavefronts per sample at 73 % of
 // the data pipe when every lane read its own corners, odd x pairs in two instructions).
 // Corners k and k + 1 (k even) differ only in x and share a line 15 times in 16, so one
@@ -26,8 +27,7 @@ __device__ __forceinline__ uint32_t pair_sample(uint32_t lane) { return (lane >>
 // instruction, the upper one of its neighbour's; the odd lane likewise.  Each then gets
 // its upper corner by a shuffle.  That is 27.7 lines per sample on the room workload's
 // rays instead of 43.7 (counted on the host); forward of 19.5 M samples 3.36 ms,
-// 3.66 before.  The corners are summed in the order k = 0 .. 7.
-// The 4 (y, z) pairs of this lane's corners (lower and upper in x) and the offsets w.
+// 3.66 before (2.82 with the groups that share the weights).
 __device__ __forceinline__ void level_corners(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
                                               float2* lo, float2* up, float* w) {
     const uint32_t N = c.res[l], Tmask = c.T - 1;
@@ -63,7 +63,8 @@ __device__ __forceinline__ void level_corners(const DevCfg& c, const float2* __r
     }
 }
 
-// Features of level l of grid position x into f[0], f[1] (whole warps, pair_sample order).
+// Features of level l of grid position x into f[0], f[1] (whole warps, pair_sample order):
+// the corners in the order k = 0 .. 7, each times its weight.
 __device__ __forceinline__ void encode_level(const DevCfg& c, const float2* __restrict__ tables, float3 x, int l,
                                              float* f) {
     float2 lo[4], up[4];
@@ -121,7 +122,7 @@ __device__ __forceinline__ void hash_encode(const DevCfg& c, const float2* __res
 // Per sample this issues 48.4 reductions in 33.3 sectors on the room workload's rays
 // (counted on the host), against 61.4 in 52.2 for sums over runs of equal cells within
 // a warp, and needs no shuffle at all: the backward of 19.5 M samples takes 4.29 ms
-// instead of 6.74.  It runs at 0.6 of the issue rate, with the integer pipe at 0.57.
+// instead of 6.74.  It issues in 0.62 of the cycles, with the integer pipe at 0.43.
 // Walks of G = 16 samples: 8 groups and 2 parities per level, two levels per warp.  With at
 // most 8 levels to scatter (G = 8): 16 groups of 8 samples, one level per warp.
 struct ScatterRole {
@@ -285,7 +286,7 @@ __device__ __forceinline__ void scatter_tile(const DevCfg& c, float2* __restrict
 // values of the 8 corners are read again (whole warps, pair_sample order: the encoding's
 // loads).  df(l): dL/df_l of this lane's sample.  The even and the odd levels are summed by
 // different warps (one thread per sample for all of them made the FP16 backward of 4.87 M
-// samples with pose terms 2.79 ms, against 1.11 without; now 2.38).
+// samples with pose terms 2.79 ms, against 1.11 without; now 2.39).
 template <class DF>
 __device__ __forceinline__ float3 hash_grad_x(const DevCfg& c, const float2* __restrict__ tables, float3 x, DF df,
                                               int l0) {

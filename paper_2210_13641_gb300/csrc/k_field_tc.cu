@@ -4,14 +4,18 @@
 // recomputing backward pass with the weight gradients accumulated in tensor memory
 // across a persistent block's tiles (steps a10-a11).
 //
-// A block owns a tile of 128 samples at a time; thread r of the block owns sample
-// row r, which is TMEM lane r of every 128-row accumulator.  Each layer is one
-// chain of tcgen05.mma instructions issued by thread 0 on shared-memory operands
-// (layout in tc_ptx.cuh), committed to an mbarrier; the block then reads the
-// accumulator rows back with tcgen05.ld, applies the activation in FP32, rounds to
-// the MLP type and writes the next operand tile.  Weight gradients are M=64
-// products over the tile's samples (MN-major operands of the same tiles) that keep
-// accumulating in TMEM until the block has no tiles left.
+// A group of 128 threads takes a tile of 128 samples through the layers: thread r of
+// the group owns operand row r, which is TMEM lane r of every 128-row accumulator.  Each
+// layer is one chain of tcgen05.mma instructions issued by an elected lane of the group's
+// first warp on shared-memory operands (layout in tc_ptx.cuh), committed to an mbarrier;
+// the group then reads the accumulator rows back with tcgen05.ld, applies the activation
+// in FP32, rounds to the MLP type and writes the next operand tile.
+// Forward: the groups of a block (six; one in a grouped render of several maps) share one
+// copy of the weights and take tiles on their own; the rows of a warp hold its samples in
+// the encoding's pair order.  Backward: a block has one such group, and two more that load
+// the tiles' inputs and scatter the table gradients; rows are in sample order.  Weight
+// gradients are M=64 products over the tile's samples (MN-major operands of the same
+// tiles) that keep accumulating in TMEM until the block has no tiles left.
 //
 // Gradient tiles are scaled by powers of two before rounding to the MLP type: the
 // colour branch (dL/dz through the colour MLP down to its input, weights W3-W5) by
@@ -472,8 +476,8 @@ __global__ void __launch_bounds__(128 * kFwdGroups, 1) k_field_fwd_tc(DevCfg c, 
 // the backward.  The features (MLP type) and dL/dfeat (FP32) of these levels travel
 // through the half of the encoding buffer that 16-bit rows leave free.  The work items are
 // taken in order of level, tile by tile.  For the floor workload (2^22 entries per
-// level, 83.6 M samples) the forward takes 19.6 ms instead of 23.4 and the backward
-// 26.0 instead of 43.3, whose random sectors came from the HBM.
+// level, 83.6 M samples) the forward takes 17.3 ms instead of 25.1 and the backward 26.5
+// instead of 44.9, whose random sectors come from the HBM.
 
 // x of sample i (0 for i >= n).
 __device__ __forceinline__ float3 position_of(const DevCfg& c, const float* __restrict__ rays, uint32_t cap,
@@ -1023,10 +1027,10 @@ __global__ void __launch_bounds__(kBwdThreads, 2) k_field_bwd_tc(DevCfg c, const
 
 // Whether a step's finest levels are taken level by level: where the tables are larger than
 // the L2.  131 k rays (10 M samples), forward + backward: at 16 levels of 2^20 entries
-// 2.0 + 2.1 ms as they are, 2.1 + 3.1 level by level; at 2^21 2.4 + 3.6 and 2.1 + 3.2, at
-// 2^22 3.0 + 5.5 and 2.5 + 3.5.  Small batches stay as they are: their two more launches
-// cost what they save (82 k samples at 2^22: 0.05 + 0.10 either way; 654 k: 0.21 + 0.36
-// and 0.18 + 0.33).
+// 2.1 + 2.3 ms as they are, 1.9 + 3.3 level by level; at 2^21 2.7 + 3.8 and 2.0 + 3.3, at
+// 2^22 3.2 + 5.6 and 2.2 + 3.5.  Small batches stay as they are: their two more launches
+// cost what they save (at 2^22, 81 k samples: 0.047 + 0.104 and 0.043 + 0.108; 322 k:
+// 0.121 + 0.208 and 0.094 + 0.223; 653 k: 0.221 + 0.364 and 0.158 + 0.340).
 bool levels_split(const DevCfg& c, uint32_t n_rays) {
     int dev = 0, l2 = 0;
     cudaGetDevice(&dev);
